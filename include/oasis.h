@@ -108,7 +108,9 @@ typedef struct oasis_params {
     int32_t spmv_variant;  /* shape of the pressure-CG product kernel (the fused Jacobi
                               iteration, or the multigrid CG product with OASIS_PC_AMG):
                               0 = autotune at solver creation (every candidate timed on
-                              this matrix, the fastest kept); k >= 1 = candidate k of
+                              this matrix, the fastest kept; where the system is small
+                              enough the whole pressure solve runs as one launch instead,
+                              which has no such shapes); k >= 1 = candidate k of
                               oasis_get_tuning */
     int32_t pressure_pc;   /* OASIS_PC_JACOBI or OASIS_PC_AMG (preconditioner of the
                               pressure CG) */
@@ -122,7 +124,9 @@ typedef struct oasis_params {
     int32_t velocity_update; /* OASIS_UPDATE_LUMPED (default) or OASIS_UPDATE_CONSISTENT */
     int32_t bicg_variant;  /* shape of the d-RHS product of the batched tentative BiCGStab:
                               0 = autotune at solver creation (every candidate timed on this
-                              mesh's pattern, the fastest kept); k >= 1 = candidate k of
+                              mesh's pattern, the fastest kept; where the system is small
+                              enough each velocity, scalar and mass solve runs as one launch
+                              instead, which has no such shapes); k >= 1 = candidate k of
                               oasis_get_tuning's bicg_* fields.  The shapes add a row's
                               products in different orders: they agree to rounding, and a
                               solver keeps its shape for its life. */
@@ -174,7 +178,8 @@ typedef struct oasis_params {
 #define OASIS_MAX_VARIANTS 16
 typedef struct oasis_tuning {
     int32_t n_variants;
-    int32_t chosen;                        /* 1-based candidate in use */
+    int32_t chosen;                        /* 1-based candidate in use (where the solve runs
+                                              as separate kernels) */
     int32_t chunk[OASIS_MAX_VARIANTS];
     int32_t min_blocks[OASIS_MAX_VARIANTS];
     int32_t prefetch[OASIS_MAX_VARIANTS];

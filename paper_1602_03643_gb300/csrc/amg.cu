@@ -179,6 +179,20 @@ HCsr smoothed_prolongator(const HCsr& F, const std::vector<int32_t>& agg, int64_
     return P;
 }
 
+// S = P - w D^-1 A P, A P given (its pattern holds P's: A has a diagonal).
+HCsr smoothed_twice(const HCsr& P, const HCsr& AP, const std::vector<double>& dinv, double w) {
+    HCsr S = AP;
+    for (int64_t i = 0; i < S.n; ++i) {
+        int64_t q = P.rp[i];
+        for (int64_t k = S.rp[i]; k < S.rp[i + 1]; ++k) {
+            S.v[k] *= -w * dinv[i];
+            while (q < P.rp[i + 1] && P.ci[q] < S.ci[k]) ++q;
+            if (q < P.rp[i + 1] && P.ci[q] == S.ci[k]) S.v[k] += P.v[q];
+        }
+    }
+    return S;
+}
+
 HCsr transpose(const HCsr& P) {
     HCsr R;
     R.n = P.m;
@@ -558,8 +572,14 @@ void amg_build(Mesh& m, cudaStream_t s) {
         L->g_a = lanes(A.nnz(), A.n);
         L->g_r = lanes(R.nnz(), R.n);
         L->g_p = lanes(P.nnz(), P.n);
+        const HCsr AP = spgemm(A, P);
+        if (m.nnz <= kResidentAmgEntries) {
+            const HCsr S = smoothed_twice(P, AP, dinv, L->omega);
+            upload_csr(L->s_rp, L->s_ci, L->s64, L->s16, S, s);
+            upload_csr(L->t_rp, L->t_ci, L->t64, L->t16, transpose(S), s);
+        }
         h->lv.push_back(std::move(L));
-        HCsr Ac = spgemm(R, spgemm(A, P));
+        HCsr Ac = spgemm(R, AP);
         A = std::move(Ac);
         const bool small = A.n <= kMaxCoarse;
         const bool stalled = (double)A.n > 0.8 * (double)h->sizes.back();

@@ -69,9 +69,20 @@ struct AmgLevelDev {
     // (levels >= 1), of R and of P, where the operator has at least
     // kSellMinRows rows (n = 0: the CSR kernels serve)
     AmgSellP sa, sr, sp;
+    // S = P - w D^-1 A P and its transpose, for the cycle of the resident solves
+    // (resident.cu; built where kResidentAmgEntries allows one)
+    DBuf<int32_t> s_rp, s_ci, t_rp, t_ci;
+    DBuf<double> s64, t64;
+    DBuf<uint16_t> s16, t16;
 };
 
 constexpr int64_t kSellMinRows = 65536;
+// Pattern entries up to which the multigrid pressure CG runs resident (one launch per
+// solve); in float64 fewer, its cycle moves twice the bytes.  Resident against separate
+// kernels, us per step at rtol 1e-8 / 1e-12 (pressure solve alone changed): 41^3 dofs,
+// 1.0 M entries: 1300 / 1519 mixed, 3132 / 3305 float64; 49^3, 1.7 M: 1705 / 1780
+// mixed; 57^3, 2.8 M: 2452 / 2032; 51^3 float64, 1.9 M: 6570 / 4893.
+constexpr int64_t kResidentAmgEntries = 1900000, kResidentAmgEntries64 = 1200000;
 
 // SELL-32 view of the finest operator (the mesh's K): the fine-level smoothers
 // read it with one lane per row, coalesced column/value loads, and 16-bit column

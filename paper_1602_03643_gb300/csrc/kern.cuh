@@ -146,6 +146,41 @@ __device__ __forceinline__ ff acc_shfl(ff a, int o) {
     return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
 }
 
+// state values as accumulators and back
+__device__ __forceinline__ double acc_of_s(double a) { return a; }
+__device__ __forceinline__ ff acc_of_s(float2 a) { return {a.x, a.y}; }
+__device__ __forceinline__ double s_of_acc(double a) { return a; }
+__device__ __forceinline__ float2 s_of_acc(ff a) { return make_float2(a.hi, a.lo); }
+
+// A product S * V added to an accumulator with the product's rounding error kept:
+// float64 exactly as before; float-float lazily (the high parts summed by an
+// error-free two-sum, every low part and error added in float, normalised once
+// by lazy_norm), about 11 float operations instead of a full float-float add's 26.
+__device__ __forceinline__ void lazy_add_prod(double& acc, double x, double v) { acc = fma(x, v, acc); }
+__device__ __forceinline__ void lazy_add_prod(ff& acc, float2 x, float v) {
+    const float p = x.x * v;
+    const float e = __fmaf_rn(x.y, v, __fmaf_rn(x.x, v, -p));
+    const ff t = two_sum(acc.hi, p);
+    acc.hi = t.hi;
+    acc.lo += t.lo + e;
+}
+__device__ __forceinline__ double lazy_norm(double a) { return a; }
+__device__ __forceinline__ ff lazy_norm(ff a) { return two_sum(a.hi, a.lo); }
+
+// S * S added lazily to an accumulator (the product's rounding error and the
+// cross terms kept, the high parts summed by an error-free two-sum, the low
+// parts in float; normalised once by lazy_norm): float64 exactly as before
+__device__ __forceinline__ void lazy_add_prod_s(double& acc, double x, double y) { acc = fma(x, y, acc); }
+__device__ __forceinline__ void lazy_add_prod_s(ff& acc, float2 x, float2 y) {
+    const float p = x.x * y.x;
+    float e = __fmaf_rn(x.x, y.x, -p);
+    e = __fmaf_rn(x.x, y.y, e);
+    e = __fmaf_rn(x.y, y.x, e);
+    const ff t = two_sum(acc.hi, p);
+    acc.hi = t.hi;
+    acc.lo += t.lo + e;
+}
+
 // Block-wide sum of NV accumulators (float-float or double), valid in thread 0.
 // Fixed shuffle/shared-memory tree: deterministic.  Any block size up to 1024.
 template <int NV, class A>

@@ -183,6 +183,7 @@ struct Solver {
                                                                        // [3 + a] scalar a
     int n_states() const { return 3 + ns; }                            // mirrored to the host each step
     RBuf partial;
+    RBuf resident;                                                     // meeting memory of the resident solves
     KrylovState* h_st = nullptr;                                       // pinned mirror [kStates]
     std::unique_ptr<StepImpl> impl;
     cudaStream_t cap[3] = {nullptr, nullptr, nullptr};

@@ -25,6 +25,7 @@
 
 #include "kern.cuh"
 #include "net.cuh"
+#include "resident.cuh"
 #include "solver.cuh"
 
 namespace oasis {
@@ -45,10 +46,6 @@ __device__ __forceinline__ typename P::V coef(double d, float f) {
     else return d;
 }
 
-__device__ __forceinline__ double acc_of_s(double a) { return a; }
-__device__ __forceinline__ ff acc_of_s(float2 a) { return {a.x, a.y}; }
-__device__ __forceinline__ double s_of_acc(double a) { return a; }
-__device__ __forceinline__ float2 s_of_acc(ff a) { return make_float2(a.hi, a.lo); }
 // S * V as an accumulator
 __device__ __forceinline__ double acc_mul_sv(double s, double v) { return s * v; }
 __device__ __forceinline__ ff acc_mul_sv(float2 s, float v) { return ff_mul_f({s.x, s.y}, v); }
@@ -402,21 +399,6 @@ __global__ void __launch_bounds__(kBlock) k_bicg_outer(StepData<P> a, int k0, Ct
     if (grid_sum<NR, Acc>(part, tot, a.partial, &a.stu->ticket) && threadIdx.x == 0)
         bicg_outer_finish<NR>(a.stu, k0, tot, ctl);
 }
-
-// A product S * V added to an accumulator with the product's rounding error kept:
-// float64 exactly as before; float-float lazily (the high parts summed by an
-// error-free two-sum, every low part and error added in float, normalised once
-// by lazy_norm), about 11 float operations instead of a full float-float add's 26.
-__device__ __forceinline__ void lazy_add_prod(double& acc, double x, double v) { acc = fma(x, v, acc); }
-__device__ __forceinline__ void lazy_add_prod(ff& acc, float2 x, float v) {
-    const float p = x.x * v;
-    const float e = __fmaf_rn(x.y, v, __fmaf_rn(x.x, v, -p));
-    const ff t = two_sum(acc.hi, p);
-    acc.hi = t.hi;
-    acc.lo += t.lo + e;
-}
-__device__ __forceinline__ double lazy_norm(double a) { return a; }
-__device__ __forceinline__ ff lazy_norm(ff a) { return two_sum(a.hi, a.lo); }
 
 // The outer sweep in row-split form (G lanes per row, U rows in flight, as the
 // row-split product): r = r0 - A Delta with float64-quality products, each
@@ -889,20 +871,6 @@ template <class P, int D>
 __global__ void __launch_bounds__(kBlock) k_tentative_velocity(StepData<P> a) {
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < a.n * D; t += (int64_t)gridDim.x * blockDim.x)
         a.uI[t] = s_add(a.u1[t], a.du[t]);
-}
-
-// S * S added lazily to an accumulator (the product's rounding error and the
-// cross terms kept, the high parts summed by an error-free two-sum, the low
-// parts in float; normalised once by lazy_norm): float64 exactly as before
-__device__ __forceinline__ void lazy_add_prod_s(double& acc, double x, double y) { acc = fma(x, y, acc); }
-__device__ __forceinline__ void lazy_add_prod_s(ff& acc, float2 x, float2 y) {
-    const float p = x.x * y.x;
-    float e = __fmaf_rn(x.x, y.x, -p);
-    e = __fmaf_rn(x.x, y.y, e);
-    e = __fmaf_rn(x.y, y.x, e);
-    const ff t = two_sum(acc.hi, p);
-    acc.hi = t.hi;
-    acc.lo += t.lo + e;
 }
 
 // The pressure right-hand side in row-split form (G lanes per row, U rows in
@@ -2339,7 +2307,9 @@ struct StepImplT final : StepImpl {
     double tune_us[OASIS_MAX_VARIANTS] = {0};
     int it_grid[OASIS_MAX_VARIANTS] = {0}, it_block[OASIS_MAX_VARIANTS] = {0};
     size_t it_smem[OASIS_MAX_VARIANTS] = {0};
-
+    ResidentPlan res_u{}, res_u1{}, res_m{}, res_p{}; // resident solves: D velocity components, one, mass, pressure
+    ResidentSync res_sync{};
+    ResidentAmg<V> res_amg{};
 
     // first multigrid CG product of a sweep, in the layout at hand
     void (*cg_first_fn() const)(StepData<P>, Ctl) {
@@ -2497,6 +2467,77 @@ struct StepImplT final : StepImpl {
         ge_red = red_grid(m.n);
         ge_nd = elem_grid(m.n * D);
         ge_c = elem_grid(m.nc);
+        res_u = resident_plan_bicg<P>(m.h_row_ptr, m.n, D);
+        res_u1 = resident_plan_bicg<P>(m.h_row_ptr, m.n, 1);
+        res_m = resident_plan_mass<P>(m.h_row_ptr, m.n, D);
+        res_p = resident_plan_cg<P>(m.h_row_ptr, m.n, Sv.prm.pressure_pc == OASIS_PC_AMG);
+        if (res_u.blocks + res_u1.blocks + res_m.blocks + res_p.blocks > 0) {
+            Sv.resident.alloc(resident_sync_bytes(m.n, sizeof(V)), nullptr);
+            OASIS_CUDA(cudaStreamSynchronize(nullptr));
+            res_sync = resident_sync(Sv.resident.p);
+        }
+        if (res_p.blocks > 0) {
+            if (Sv.prm.pressure_pc == OASIS_PC_AMG) res_amg = resident_amg();
+            else a.au = reinterpret_cast<V*>(a.pq0);   // u of the float64 Jacobi form
+        }
+    }
+
+    // The hierarchy and this solver's cycle vectors as the resident solve reads them.
+    ResidentAmg<V> resident_amg() const {
+        const AmgHierarchy& H = *Sv.m->amg;
+        ResidentAmg<V> r;
+        r.levels = (int32_t)H.lv.size();
+        r.nc = (int32_t)H.nc;
+        r.ld = (int32_t)H.ld;
+        if constexpr (P::mixed) r.inv = H.inv32.p;
+        else r.inv = H.inv64.p;
+        auto vec = [](const DBuf<double>& b) { return reinterpret_cast<V*>(b.p); };
+        r.rc = vec(Sv.amgw.rin[r.levels]);
+        r.xc = vec(Sv.amgw.xo[r.levels]);
+        auto lanes = [&](int64_t rows, size_t nnz) {
+            // as many lanes per row as there are threads and entries for
+            const double mean = (double)nnz / (double)std::max<int64_t>(1, rows);
+            const int64_t per_block = (rows + res_p.blocks - 1) / res_p.blocks;
+            int g = 32;
+            while (g > 1 && (per_block * g > res_p.threads || g > mean)) g /= 2;
+            return g;
+        };
+        for (int l = 0; l < r.levels; ++l) {
+            const AmgLevelDev& v = *H.lv[l];
+            ResidentLevel<V>& o = r.lv[l];
+            o.n = (int32_t)v.n;
+            o.w = (V)v.omega;
+            o.a_rp = v.rp;
+            o.a_ci = v.ci;
+            o.s_rp = v.s_rp.p;
+            o.s_ci = v.s_ci.p;
+            o.t_rp = v.t_rp.p;
+            o.t_ci = v.t_ci.p;
+            if constexpr (P::mixed) {
+                o.d = v.d32.p;
+                o.a = v.a16;
+                o.s = v.s16.p;
+                o.t = v.t16.p;
+            } else {
+                o.d = v.d64.p;
+                o.a = v.a64;
+                o.s = v.s64.p;
+                o.t = v.t64.p;
+            }
+            o.r = l == 0 ? a.ar : vec(Sv.amgw.rin[l]);
+            o.x = l == 0 ? a.au : vec(Sv.amgw.xo[l]);
+            o.y = vec(Sv.amgw.x[l]);
+            o.ga = lanes(v.n, (size_t)v.nnz);
+            o.gs = lanes(v.n, v.s16.n);
+            o.gt = lanes(l + 1 < r.levels ? H.lv[l + 1]->n : H.nc, v.s16.n);
+        }
+        return r;
+    }
+
+    // Whether a solve with this plan runs resident: not where the caller forces a
+    // product shape or times kernel families (eager profiling).
+    bool resident(const ResidentPlan& pl, int32_t forced) const {
+        return pl.blocks > 0 && forced == 0 && !(Sv.prof_on && !Sv.prm.use_graph);
     }
 
     void assemble(cudaStream_t s) override {
@@ -2542,6 +2583,11 @@ struct StepImplT final : StepImpl {
     // BiCGStab with refinement sweeps on the system of q (state index `which`).
     template <int DD, int NR>
     void bicg_run(const StepData<P>& q, cudaStream_t s, int which, int k0, bool graph) {
+        const ResidentPlan& pl = NR == 1 ? res_u1 : res_u;
+        if (resident(pl, Sv.prm.bicg_variant)) {
+            resident_bicg<P, DD, NR>(q, k0, ctl_u(Loop{}), pl, res_sync, s);
+            return;
+        }
         const BicgGrids G = bicg_grids<DD, NR>();
         Sv.run_loops(
             s, graph, which,
@@ -2667,6 +2713,10 @@ struct StepImplT final : StepImpl {
         Sv.prof_end(s, pg);
         k_phi_guess<P><<<ge_n, kBlock, 0, s>>>(a, mode);
         OASIS_CUDA(cudaGetLastError());
+        if (resident(res_p, Sv.prm.spmv_variant)) {
+            resident_cg<P>(a, ctl_p(Loop{}), res_amg, res_p, res_sync, s);
+            return;
+        }
         if (Sv.prm.pressure_pc == OASIS_PC_AMG) {
             const AmgHierarchy& H = *Sv.m->amg;
             ProfHook hook;
@@ -2755,7 +2805,8 @@ struct StepImplT final : StepImpl {
 
     void update(cudaStream_t s, bool graph) override {
         if (Sv.prm.velocity_update == OASIS_UPDATE_CONSISTENT) {
-            Sv.run_single(
+            if (resident(res_m, Sv.prm.bicg_variant)) resident_mass<P, D>(a, Sv.prm.dt, ctl_m(Loop{}), res_m, res_sync, s);
+            else Sv.run_single(
                 s, graph, 2,
                 [&](cudaStream_t ss, const Loop& lp) {
                     const int pm = Sv.prof_begin(ss, OASIS_PROF_MASS);
