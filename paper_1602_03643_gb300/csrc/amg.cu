@@ -13,6 +13,7 @@
 #include <cuda_bf16.h>
 
 #include "amg.cuh"
+#include "resident.cuh"
 #include "solver.cuh"
 
 namespace oasis {
@@ -573,7 +574,7 @@ void amg_build(Mesh& m, cudaStream_t s) {
         L->g_r = lanes(R.nnz(), R.n);
         L->g_p = lanes(P.nnz(), P.n);
         const HCsr AP = spgemm(A, P);
-        if (m.nnz <= kResidentAmgEntries) {
+        if (m.nnz <= kResidentAmgEntries || (!h->lv.empty() && A.n <= kTailRows)) {
             const HCsr S = smoothed_twice(P, AP, dinv, L->omega);
             upload_csr(L->s_rp, L->s_ci, L->s64, L->s16, S, s);
             upload_csr(L->t_rp, L->t_ci, L->t64, L->t16, transpose(S), s);
@@ -619,6 +620,8 @@ void AmgWork::alloc(const AmgHierarchy& h, size_t vbytes) {
         rin[l].alloc(cnt);
         if (l == L) OASIS_CUDA(cudaMemset(rin[l].p, 0, rin[l].bytes()));
     }
+    meet.alloc(resident_sync_bytes(0, 0));
+    OASIS_CUDA(cudaMemset(meet.p, 0, meet.bytes()));
 }
 
 // ------------------------------------------------------------------ kernels
@@ -663,21 +666,20 @@ struct AmgRowArgs {
     const int32_t* __restrict__ rp;
     const int32_t* __restrict__ ci;
     const AV* __restrict__ a;
-    const V* __restrict__ d;     // 1 / a_ii (smoothing)
-    V w;                         // Jacobi weight (smoothing)
+    const V* __restrict__ d;     // 1 / a_ii (post; restriction: of the next level, or null)
+    V w;                         // Jacobi weight (likewise)
     const V* __restrict__ r;     // right-hand side of the level (smoothing)
-    const V* __restrict__ x;     // post: the iterate
-    const V* __restrict__ v;     // transfers: the vector multiplied
-    V* __restrict__ out;         // pre: x; post: the smoothed iterate; transfers: y
-    V* __restrict__ res;         // pre: the residual
+    const V* __restrict__ x;     // smoothing: the iterate; transfers: the vector multiplied
+    V* __restrict__ out;         // post: the smoothed iterate; transfers: y
+    V* __restrict__ res;         // pre: the residual; restriction: w D^-1 y of the next level
     const KrylovState* st;
 };
 
-// MODE kRowPre:      x = w D^-1 r, res = r - A x (smoothing from zero; the gathered
-//                    operand is w d_j r_j);
+// MODE kRowPre:      res = r - A x, x = w D^-1 r the sweep from zero (written with r, by
+//                    the restriction: one value gathered per entry, not d_j and r_j);
 //      kRowPost:     out = x + w D^-1 (r - A x);
-//      kRowProlong:  out += P v;
-//      kRowRestrict: out = R v.
+//      kRowProlong:  out += P x;
+//      kRowRestrict: out = R x, and the next level's sweep from zero, res = w D^-1 out.
 template <class V, class AV, int G, int U, int MODE>
 __device__ __forceinline__ void amg_rows(const AmgRowArgs<V, AV>& p) {
     if (amg_done(p.st)) return;
@@ -712,9 +714,7 @@ __device__ __forceinline__ void amg_rows(const AmgRowArgs<V, AV>& p) {
             V g[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                if constexpr (MODE == kRowPre) g[u] = p.w * p.d[j[u]] * p.r[j[u]];
-                else if constexpr (MODE == kRowPost) g[u] = p.x[j[u]];
-                else g[u] = p.v[j[u]];
+                g[u] = p.x[j[u]];
             }
             more = false;
 #pragma unroll
@@ -733,13 +733,13 @@ __device__ __forceinline__ void amg_rows(const AmgRowArgs<V, AV>& p) {
                 const int64_t ii = i[u];
                 if constexpr (MODE == kRowPre) {
                     p.res[ii] = p.r[ii] - t;
-                    p.out[ii] = p.w * p.d[ii] * p.r[ii];
                 } else if constexpr (MODE == kRowPost) {
                     p.out[ii] = p.x[ii] + p.w * p.d[ii] * (p.r[ii] - t);
                 } else if constexpr (MODE == kRowProlong) {
                     p.out[ii] = p.out[ii] + t;
                 } else {
                     p.out[ii] = t;
+                    if (p.d) p.res[ii] = p.w * p.d[ii] * t;
                 }
             }
         }
@@ -785,8 +785,9 @@ __device__ __forceinline__ int32_t fine_col(const AmgSellView& F, int64_t q, int
     }
 }
 
-// PRE: x = w D^-1 r and res = r - A x (smoothing from zero); else
-// out = x + w D^-1 (r - A x).  The gathered operand is w d_j r_j (PRE) or x_j.
+// PRE: res = r - A x, x = w D^-1 r the sweep from zero (written by the CG's vector
+// update: one value gathered per entry, not d_j and r_j; random dof order, float64,
+// 383,542 rows: 37.2 -> 28.0 us per sweep); else out = x + w D^-1 (r - A x).
 // (Two slices per warp in flight were measured slower at 128^3: 61 against
 // 47 us per sweep, the extra registers costing more resident warps than the
 // second chain gains.)
@@ -820,7 +821,7 @@ __global__ void __launch_bounds__(kBlock) k_amg_fine(AmgSellView F, const AV* __
             }
             V g[C];
 #pragma unroll
-            for (int u = 0; u < C; ++u) g[u] = PRE ? w * d[j[u]] * r[j[u]] : x[j[u]];
+            for (int u = 0; u < C; ++u) g[u] = x[j[u]];
 #pragma unroll
             for (int u = 0; u < C; ++u)
                 if (k + u < len) s += kv[u] * g[u];
@@ -828,7 +829,6 @@ __global__ void __launch_bounds__(kBlock) k_amg_fine(AmgSellView F, const AV* __
         if (i < F.n) {
             if constexpr (PRE) {
                 res[i] = r[i] - s;
-                out[i] = w * d[i] * r[i];
             } else {
                 out[i] = x[i] + w * d[i] * (r[i] - s);
             }
@@ -876,7 +876,7 @@ __global__ void __launch_bounds__(kBlock) k_amg_fine_pairs(AmgSellView F, const 
                 int32_t j = row + (int32_t)(int16_t)half;
                 j = j < 0 ? j + n32 : j;
                 j = j >= n32 ? j - n32 : j;
-                g[e] = PRE ? w * d[j] * r[j] : x[j];
+                g[e] = x[j];
             }
 #pragma unroll
             for (int u = 0; u < C2; ++u)
@@ -888,7 +888,6 @@ __global__ void __launch_bounds__(kBlock) k_amg_fine_pairs(AmgSellView F, const 
         if (i < F.n) {
             if constexpr (PRE) {
                 res[i] = r[i] - sum;
-                out[i] = w * d[i] * r[i];
             } else {
                 out[i] = x[i] + w * d[i] * (r[i] - sum);
             }
@@ -907,8 +906,8 @@ struct SellPView {
 };
 
 // Row kernels of the float32 cycle on a pair-packed SELL-32 operator, the modes
-// of amg_rows (pre: x = w D^-1 r, res = r - A x; post: out = src + w D^-1 (r - A src);
-// prolong: out += P src; restrict: out = R src).  SP warps serve one slice: warp
+// of amg_rows (pre: res = r - A src; post: out = src + w D^-1 (r - A src);
+// prolong: out += P src; restrict: out = R src, res = w D^-1 out where d is given).  SP warps serve one slice: warp
 // p of the slice takes the rounds p, p + SP, ... of C2 words each; per round it
 // loads C2 words of values and C2 of offsets (W: C2 pairs of whole columns) per
 // lane (2 C2 entries), then their 2 C2 gathers, and adds the products in entry
@@ -953,8 +952,7 @@ __global__ void __launch_bounds__(kBlock) k_amg_sellp(SellPView S, const float* 
 #pragma unroll
                 for (int e = 0; e < 2 * C2; ++e) {
                     const int32_t j = h.z + (int32_t)((e & 1) ? cw[e >> 1].y : cw[e >> 1].x);
-                    if constexpr (MODE == kRowPre) g[e] = w * d[j] * r[j];
-                    else g[e] = src[j];
+                    g[e] = src[j];
                 }
 #pragma unroll
                 for (int u = 0; u < C2; ++u)
@@ -978,16 +976,24 @@ __global__ void __launch_bounds__(kBlock) k_amg_sellp(SellPView S, const float* 
         if (sub == 0 && sl < S.n_slices && i < S.n) {
             if constexpr (MODE == kRowPre) {
                 res[i] = r[i] - sum;
-                out[i] = w * d[i] * r[i];
             } else if constexpr (MODE == kRowPost) {
                 out[i] = src[i] + w * d[i] * (r[i] - sum);
             } else if constexpr (MODE == kRowProlong) {
                 out[i] = out[i] + sum;
             } else {
                 out[i] = sum;
+                if (d) res[i] = w * d[i] * sum;
             }
         }
     }
+}
+
+// z = w D^-1 r
+template <class V>
+__global__ void __launch_bounds__(kBlock) k_amg_scale(int64_t n, V w, const V* __restrict__ d, const V* __restrict__ r,
+                                                      V* __restrict__ z) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        z[i] = w * d[i] * r[i];
 }
 
 // coarsest level: x = inv r with inv dense and row-major, leading dimension ld
@@ -1128,9 +1134,12 @@ void launch_sellp(const AmgSellP& A, const float* d, float w, const float* r, co
     }
 
 template <class V>
-void amg_vcycle(const AmgHierarchy& h, AmgWork& wk, const V* r, V* u, const KrylovState* st, cudaStream_t s,
+void amg_vcycle(const AmgHierarchy& h, AmgWork& wk, const V* r, V* u, KrylovState* st, cudaStream_t s, bool smoothed,
                 const ProfHook* prof) {
     const int L = (int)h.lv.size();
+    // levels tail .. L - 1 and the dense one run in the tail's launch
+    int tail = 1;
+    while (tail < L && h.lv[tail]->n > kTailRows) ++tail;
     // the pair-packed copies serve the float32 cycle only
     auto sellp_ok = [](const AmgSellP& A) { return sizeof(V) == 4 && A.n > 0; };
     int ph = -1;
@@ -1142,76 +1151,79 @@ void amg_vcycle(const AmgHierarchy& h, AmgWork& wk, const V* r, V* u, const Kryl
     };
     using AV = StoredT<V>;
     auto vec = [](DBuf<double>& b) { return reinterpret_cast<V*>(b.p); };
+    auto w_of = [&](int l) { return (V)h.lv[l]->omega; };
+    auto d_of = [&](int l) { return pick<V>(h.lv[l]->d32.p, h.lv[l]->d64.p); };
     // level inputs: rin[0] = r; outputs: xo[0] = u
     auto rin = [&](int l) -> const V* { return l == 0 ? r : vec(wk.rin[l]); };
     auto xo = [&](int l) -> V* { return l == 0 ? u : vec(wk.xo[l]); };
-    for (int l = 0; l < L; ++l) {
+    if (!smoothed)
+        k_amg_scale<V><<<(int)std::min<int64_t>((h.lv[0]->n + kBlock - 1) / kBlock, 4096), kBlock, 0, s>>>(
+            h.lv[0]->n, w_of(0), d_of(0), r, vec(wk.x[0]));
+    for (int l = 0; l < tail; ++l) {
         const AmgLevelDev& lv = *h.lv[l];
-        const AV* a = stored<V>(lv.a16, lv.a64);
-        const V* d = pick<V>(lv.d32.p, lv.d64.p);
-        const V w = (V)lv.omega;
         if (l == 0) {
             pbeg(OASIS_PROF_AMG_FINE);
-            launch_fine<V, true>(h.fine, d, w, rin(0), nullptr, vec(wk.x[0]), vec(wk.res[0]), st, s);
+            launch_fine<V, true>(h.fine, d_of(0), w_of(0), r, vec(wk.x[0]), nullptr, vec(wk.res[0]), st, s);
             pend();
         } else {
             pbeg(OASIS_PROF_AMG_COARSE);
             if (sellp_ok(lv.sa)) {
                 if constexpr (sizeof(V) == 4)
-                    launch_sellp<kRowPre>(lv.sa, d, w, rin(l), nullptr, vec(wk.x[l]), vec(wk.res[l]), st, s);
+                    launch_sellp<kRowPre>(lv.sa, d_of(l), w_of(l), rin(l), vec(wk.x[l]), nullptr, vec(wk.res[l]), st, s);
             } else {
-                AmgRowArgs<V, AV> ra{lv.n, lv.rp, lv.ci, a, d, w, rin(l), nullptr, nullptr, vec(wk.x[l]),
-                                     vec(wk.res[l]), st};
+                AmgRowArgs<V, AV> ra{lv.n, lv.rp, lv.ci, stored<V>(lv.a16, lv.a64), nullptr, V(0), rin(l), vec(wk.x[l]),
+                                     nullptr, vec(wk.res[l]), st};
                 AMG_DISPATCH(lv.g_a, k_amg_pre, lv.n, ra);
             }
             pend();
         }
+        // restriction, with the next level's sweep from zero where it is one of these
         const int64_t nc = l + 1 < L ? h.lv[l + 1]->n : h.nc;
-        const AV* rv = stored<V>(lv.r16.p, lv.r64.p);
+        const V* nd = l + 1 < tail ? d_of(l + 1) : nullptr;
+        const V nw = l + 1 < tail ? w_of(l + 1) : V(0);
         pbeg(OASIS_PROF_AMG_TRANSFER);
         if (sellp_ok(lv.sr)) {
             if constexpr (sizeof(V) == 4)
-                launch_sellp<kRowRestrict>(lv.sr, nullptr, 0.f, nullptr, vec(wk.res[l]), vec(wk.rin[l + 1]), nullptr,
-                                           st, s);
+                launch_sellp<kRowRestrict>(lv.sr, nd, nw, nullptr, vec(wk.res[l]), vec(wk.rin[l + 1]),
+                                           vec(wk.x[l + 1]), st, s);
         } else {
-            AmgRowArgs<V, AV> rr{nc, lv.r_rp.p, lv.r_ci.p, rv, nullptr, V(0), nullptr, nullptr, vec(wk.res[l]),
-                                 vec(wk.rin[l + 1]), nullptr, st};
+            AmgRowArgs<V, AV> rr{nc, lv.r_rp.p, lv.r_ci.p, stored<V>(lv.r16.p, lv.r64.p), nd, nw, nullptr,
+                                 vec(wk.res[l]), vec(wk.rin[l + 1]), vec(wk.x[l + 1]), st};
             AMG_DISPATCH(lv.g_r, k_amg_restrict, nc, rr);
         }
         pend();
     }
     pbeg(OASIS_PROF_AMG_COARSE);
-    k_amg_dense<V><<<(int)std::max<int64_t>(1, h.nc), kDenseBlock, 0, s>>>(h.nc, h.ld, pick<V>(h.inv32.p, h.inv64.p),
-                                                                     vec(wk.rin[L]),
-                                                         vec(wk.xo[L]), st);
+    if (tail < L)
+        resident_tail<V>(h, wk, tail, st, s);
+    else
+        k_amg_dense<V><<<(int)std::max<int64_t>(1, h.nc), kDenseBlock, 0, s>>>(
+            h.nc, h.ld, pick<V>(h.inv32.p, h.inv64.p), vec(wk.rin[L]), vec(wk.xo[L]), st);
     pend();
-    for (int l = L - 1; l >= 0; --l) {
+    for (int l = tail - 1; l >= 0; --l) {
         const AmgLevelDev& lv = *h.lv[l];
-        const AV* a = stored<V>(lv.a16, lv.a64);
-        const V* d = pick<V>(lv.d32.p, lv.d64.p);
-        const V w = (V)lv.omega;
-        const AV* pv = stored<V>(lv.p16.p, lv.p64.p);
         pbeg(OASIS_PROF_AMG_TRANSFER);
         if (sellp_ok(lv.sp)) {
             if constexpr (sizeof(V) == 4)
                 launch_sellp<kRowProlong>(lv.sp, nullptr, 0.f, nullptr, xo(l + 1), vec(wk.x[l]), nullptr, st, s);
         } else {
-            AmgRowArgs<V, AV> pr{lv.n, lv.p_rp.p, lv.p_ci.p, pv, nullptr, V(0), nullptr, nullptr, xo(l + 1),
-                                 vec(wk.x[l]), nullptr, st};
+            AmgRowArgs<V, AV> pr{lv.n, lv.p_rp.p, lv.p_ci.p, stored<V>(lv.p16.p, lv.p64.p), nullptr, V(0), nullptr,
+                                 xo(l + 1), vec(wk.x[l]), nullptr, st};
             AMG_DISPATCH(lv.g_p, k_amg_prolong, lv.n, pr);
         }
         pend();
         if (l == 0) {
             pbeg(OASIS_PROF_AMG_FINE);
-            launch_fine<V, false>(h.fine, d, w, rin(0), vec(wk.x[0]), xo(0), nullptr, st, s);
+            launch_fine<V, false>(h.fine, d_of(0), w_of(0), r, vec(wk.x[0]), u, nullptr, st, s);
             pend();
         } else {
             pbeg(OASIS_PROF_AMG_COARSE);
             if (sellp_ok(lv.sa)) {
                 if constexpr (sizeof(V) == 4)
-                    launch_sellp<kRowPost>(lv.sa, d, w, rin(l), vec(wk.x[l]), xo(l), nullptr, st, s);
+                    launch_sellp<kRowPost>(lv.sa, d_of(l), w_of(l), rin(l), vec(wk.x[l]), xo(l), nullptr, st, s);
             } else {
-                AmgRowArgs<V, AV> po{lv.n, lv.rp, lv.ci, a, d, w, rin(l), vec(wk.x[l]), nullptr, xo(l), nullptr, st};
+                AmgRowArgs<V, AV> po{lv.n, lv.rp, lv.ci, stored<V>(lv.a16, lv.a64), d_of(l), w_of(l), rin(l),
+                                     vec(wk.x[l]), xo(l), nullptr, st};
                 AMG_DISPATCH(lv.g_a, k_amg_post, lv.n, po);
             }
             pend();
@@ -1222,9 +1234,9 @@ void amg_vcycle(const AmgHierarchy& h, AmgWork& wk, const V* r, V* u, const Kryl
 #undef AMG_DISPATCH
 #undef AMG_LAUNCH
 
-template void amg_vcycle<float>(const AmgHierarchy&, AmgWork&, const float*, float*, const KrylovState*, cudaStream_t,
+template void amg_vcycle<float>(const AmgHierarchy&, AmgWork&, const float*, float*, KrylovState*, cudaStream_t, bool,
                                 const ProfHook*);
-template void amg_vcycle<double>(const AmgHierarchy&, AmgWork&, const double*, double*, const KrylovState*,
-                                 cudaStream_t, const ProfHook*);
+template void amg_vcycle<double>(const AmgHierarchy&, AmgWork&, const double*, double*, KrylovState*, cudaStream_t,
+                                 bool, const ProfHook*);
 
 }  // namespace oasis

@@ -70,7 +70,8 @@ struct AmgLevelDev {
     // kSellMinRows rows (n = 0: the CSR kernels serve)
     AmgSellP sa, sr, sp;
     // S = P - w D^-1 A P and its transpose, for the cycle of the resident solves
-    // (resident.cu; built where kResidentAmgEntries allows one)
+    // (resident.cu; built where kResidentAmgEntries allows one, and for the levels of
+    // the cycle's tail)
     DBuf<int32_t> s_rp, s_ci, t_rp, t_ci;
     DBuf<double> s64, t64;
     DBuf<uint16_t> s16, t16;
@@ -83,6 +84,12 @@ constexpr int64_t kSellMinRows = 65536;
 // 1.0 M entries: 1300 / 1519 mixed, 3132 / 3305 float64; 49^3, 1.7 M: 1705 / 1780
 // mixed; 57^3, 2.8 M: 2452 / 2032; 51^3 float64, 1.9 M: 6570 / 4893.
 constexpr int64_t kResidentAmgEntries = 1900000, kResidentAmgEntries64 = 1200000;
+// The tail of a V-cycle of separate kernels, from the first coarser level with at most
+// this many rows down to the dense one and back, is one resident launch (resident.cu).
+// us per two steps with 20,000 / 40,000 / 60,000: 73x71x74 dofs float64 (level 1: 35k
+// rows) 20573 / 19734 / 19697; channel 128x96x96 (53k) 21021 / 21077 / 21261; per three
+// steps of 64^3 mixed (35k) 6330 / 6379 / 6372.
+constexpr int64_t kTailRows = 40000;
 
 // SELL-32 view of the finest operator (the mesh's K): the fine-level smoothers
 // read it with one lane per row, coalesced column/value loads, and 16-bit column
@@ -133,8 +140,13 @@ void amg_build(Mesh& m, cudaStream_t s);
 // Per-solver work vectors of the V-cycle.
 struct AmgWork {
     std::vector<DBuf<double>> x, xo, res, rin;   // raw storage; viewed as V
+    DBuf<unsigned char> meet;                    // where the tail's blocks meet
     void alloc(const AmgHierarchy& h, size_t vbytes);
 };
+
+// The cycle's tail from level `first` (rin[first] -> xo[first]); resident.cu.
+template <class V>
+void resident_tail(const AmgHierarchy& h, AmgWork& w, int first, KrylovState* st, cudaStream_t s);
 
 // Optional timing of the V-cycle's kernels by family (eager profiling): begin
 // returns a handle that end closes; both are no-ops when the hook is absent.
@@ -146,8 +158,9 @@ struct ProfHook {
 
 // u = M r with one V(1,1) cycle (device arrays of n_0 values of type V).  The
 // kernels return at once when `done` (the CG's col_done / in_done flags) is set.
+// smoothed: w.x[0] holds w D^-1 r already (the CG's vector update writes it).
 template <class V>
-void amg_vcycle(const AmgHierarchy& h, AmgWork& w, const V* r, V* u, const KrylovState* st, cudaStream_t s,
+void amg_vcycle(const AmgHierarchy& h, AmgWork& w, const V* r, V* u, KrylovState* st, cudaStream_t s, bool smoothed,
                 const ProfHook* prof = nullptr);
 
 }  // namespace oasis

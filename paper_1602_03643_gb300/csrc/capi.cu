@@ -252,7 +252,8 @@ static Solver* create_solver(Mesh* m, const oasis_params* prm, int64_t n_dir, co
     S->beta.alloc(vb * m->nc * 4, s);
     if (prm->convection == OASIS_CONV_ABE) S->beta2.alloc(vb * m->nc * 4, s);
     else S->ubar.alloc(vb * n * D, s);
-    for (auto& w : S->w) w.alloc(vb * n * D, s);
+    // ph and sh (6, 7) hold padded records (Pub, kern.cuh)
+    for (int q = 0; q < 9; ++q) S->w[q].alloc(vb * n * (D == 3 && (q == 6 || q == 7) ? 4 : D), s);
     for (auto& w : S->pw) w.alloc(vb * n, s);
     for (auto& q : S->pq) q.alloc(4 * vb * n, s);
     if (prm->velocity_update == OASIS_UPDATE_CONSISTENT)

@@ -472,11 +472,33 @@ struct Vec {
     T v[N];
 };
 
+// NR components of a dof as neighbours gather them: one aligned record (three
+// components padded to four), so that a neighbour costs one vector load and, in
+// float64, one 32-byte sector where a 24-byte record lies across two.
+template <class V, int NR>
+struct alignas((NR == 1 ? 1 : NR == 2 ? 2 : sizeof(V) == 4 ? 4 : 2) * sizeof(V)) Pub {
+    V v[NR == 3 ? 4 : NR];
+};
+
 // Four values loaded or stored as one aligned vector access.
 template <class T>
 struct alignas(4 * sizeof(T)) Vec4A {
     T v[4];
 };
+
+// 16 bytes of values (arrays from the device allocator, indexed in whole packs).
+template <class V>
+struct alignas(16) Pack {
+    V v[16 / sizeof(V)];
+};
+template <class V>
+__device__ __forceinline__ Pack<V> pack_load(const V* __restrict__ a, int64_t t) {
+    return reinterpret_cast<const Pack<V>*>(a)[t];
+}
+template <class V>
+__device__ __forceinline__ void pack_store(V* __restrict__ a, int64_t t, const Pack<V>& p) {
+    reinterpret_cast<Pack<V>*>(a)[t] = p;
+}
 
 // Entry phase of a tile with U entries per thread in flight: `load(e)` reads
 // everything an entry needs (its value, column and gathered vector entries) into

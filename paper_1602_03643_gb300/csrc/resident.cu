@@ -429,12 +429,6 @@ struct BicgScalars {
     int it_total[NR], col_done[NR], in_done[NR], act[NR], status;
 };
 
-// NR components of a dof as neighbours gather them: one aligned load.
-template <class V, int NR>
-struct alignas((NR == 1 ? 1 : NR == 2 ? 2 : sizeof(V) == 4 ? 4 : 2) * sizeof(V)) Pub {
-    V v[NR == 3 ? 4 : NR];
-};
-
 // Right-preconditioned BiCGStab with Jacobi inside refinement sweeps: the method,
 // the stopping tests and the counters of the separate kernels (k_bicg_*, step.cu).
 // Per iteration the blocks meet three times (mixed) or four (float64): after p and
@@ -819,6 +813,22 @@ __device__ __forceinline__ bool res_vcycle(GridMeet& gm, const ResidentAmg<V>& m
         if (!level_rows<V, kLevelProlong>(L.gs, up, gm.m.count, gm.next())) return false;
     }
     return true;
+}
+
+// The tail of a V-cycle of separate kernels: the small levels' kernels took 3.5-5 us
+// each whatever their size; one launch with two meetings per level takes ~2.5 us per
+// meeting.
+template <class V>
+__global__ void __launch_bounds__(512, 1) k_resident_tail(ResidentAmg<V> m, KrylovState* st, ResidentSync sy) {
+    if (st->col_done[0] || st->in_done[0]) return;
+    GridMeet gm(sy);
+    const bool ok = res_vcycle<V>(gm, m, true, [&](V w, V* y) {
+        const ResidentLevel<V>& L = m.lv[0];
+        const LevelArgs<V> smooth{L.n, L.a_rp, L.a_ci, L.a, L.r, nullptr, L.d, w, y};
+        level_rows<V, kLevelSmooth>(L.ga, smooth, nullptr, 0u);
+    });
+    if (!ok && threadIdx.x == 0) st->status = OASIS_EWAIT;
+    gm.leave();
 }
 
 // How the pressure CG is preconditioned and how its iteration is arranged.
@@ -1374,10 +1384,12 @@ constexpr int res_static(bool mass) {
 
 template <class... KArgs, class... Args>
 void launch(void (*fn)(KArgs...), const ResidentPlan& pl, cudaStream_t s, Args&&... args) {
-    cudaFuncAttributes fa{};
-    OASIS_CUDA(cudaFuncGetAttributes(&fa, fn));
-    OASIS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    smem_optin() - (int)fa.sharedSizeBytes));
+    if (pl.smem > 0) {
+        cudaFuncAttributes fa{};
+        OASIS_CUDA(cudaFuncGetAttributes(&fa, fn));
+        OASIS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        smem_optin() - (int)fa.sharedSizeBytes));
+    }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)pl.blocks);
     cfg.blockDim = dim3((unsigned)pl.threads);
@@ -1488,6 +1500,71 @@ void resident_mass(const StepData<P>& q, double dt, const Ctl& c, const Resident
 #undef OASIS_RES_LAUNCH
 }
 #undef OASIS_RES_SHAPE
+
+template <class V>
+ResidentAmg<V> resident_amg(const AmgHierarchy& h, AmgWork& w, int first, int blocks, int threads) {
+    ResidentAmg<V> r;
+    const int L = (int)h.lv.size();
+    r.levels = L - first;
+    r.nc = (int32_t)h.nc;
+    r.ld = (int32_t)h.ld;
+    if constexpr (sizeof(V) == 4) r.inv = h.inv32.p;
+    else r.inv = h.inv64.p;
+    auto vec = [](const DBuf<double>& b) { return reinterpret_cast<V*>(b.p); };
+    r.rc = vec(w.rin[L]);
+    r.xc = vec(w.xo[L]);
+    auto lanes = [&](int64_t rows, size_t nnz) {
+        // as many lanes per row as there are threads and entries for
+        const double mean = (double)nnz / (double)std::max<int64_t>(1, rows);
+        const int64_t per_block = (rows + blocks - 1) / blocks;
+        int g = 32;
+        while (g > 1 && (per_block * g > threads || g > mean)) g /= 2;
+        return g;
+    };
+    for (int l = first; l < L; ++l) {
+        const AmgLevelDev& v = *h.lv[l];
+        ResidentLevel<V>& o = r.lv[l - first];
+        o.n = (int32_t)v.n;
+        o.w = (V)v.omega;
+        o.a_rp = v.rp;
+        o.a_ci = v.ci;
+        o.s_rp = v.s_rp.p;
+        o.s_ci = v.s_ci.p;
+        o.t_rp = v.t_rp.p;
+        o.t_ci = v.t_ci.p;
+        if constexpr (sizeof(V) == 4) {
+            o.d = v.d32.p;
+            o.a = v.a16;
+            o.s = v.s16.p;
+            o.t = v.t16.p;
+        } else {
+            o.d = v.d64.p;
+            o.a = v.a64;
+            o.s = v.s64.p;
+            o.t = v.t64.p;
+        }
+        o.r = vec(w.rin[l]);
+        o.x = vec(w.xo[l]);
+        o.y = vec(w.x[l]);
+        o.ga = lanes(v.n, (size_t)v.nnz);
+        o.gs = lanes(v.n, v.s16.n);
+        o.gt = lanes(l + 1 < L ? h.lv[l + 1]->n : h.nc, v.s16.n);
+    }
+    return r;
+}
+
+template <class V>
+void resident_tail(const AmgHierarchy& h, AmgWork& w, int first, KrylovState* st, cudaStream_t s) {
+    ResidentPlan pl;
+    pl.threads = 512;
+    // at least 16 rows of the tail's finest level per block
+    pl.blocks = (int)std::max<int64_t>(1, std::min<int64_t>(num_sms(), (h.lv[first]->n + 15) / 16));
+    launch(k_resident_tail<V>, pl, s, resident_amg<V>(h, w, first, pl.blocks, pl.threads), st, resident_sync(w.meet.p));
+}
+template void resident_tail<float>(const AmgHierarchy&, AmgWork&, int, KrylovState*, cudaStream_t);
+template void resident_tail<double>(const AmgHierarchy&, AmgWork&, int, KrylovState*, cudaStream_t);
+template ResidentAmg<float> resident_amg<float>(const AmgHierarchy&, AmgWork&, int, int, int);
+template ResidentAmg<double> resident_amg<double>(const AmgHierarchy&, AmgWork&, int, int, int);
 
 #define OASIS_RES(P)                                                                                             \
     template void resident_bicg<P, 3, 3>(const StepData<P>&, int, const Ctl&, const ResidentPlan&,               \

@@ -64,6 +64,11 @@ struct ResidentAmg {
     ResidentLevel<V> lv[kResLevels];
 };
 
+// The hierarchy from level `first` on, and a solver's cycle vectors, for a launch of
+// the given shape.
+template <class V>
+ResidentAmg<V> resident_amg(const AmgHierarchy& h, AmgWork& w, int first, int blocks, int threads);
+
 // D components per dof, NR of them (from k0) solved together.
 template <class P, int D, int NR>
 void resident_bicg(const StepData<P>& q, int k0, const Ctl& c, const ResidentPlan& pl, const ResidentSync& sy,

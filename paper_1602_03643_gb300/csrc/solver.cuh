@@ -68,6 +68,9 @@ struct StepData {
     CgQuad<V> *pq0, *pq1;
     V *pp, *pdl, *xv;
     V *ar, *as, *aw, *au;             // multigrid-preconditioned CG: r, s, w = K u, u = M r
+    V* az;                            // z = w D^-1 r of the finest multigrid level, and its w and D^-1
+    const V* ad0;
+    V aw0;
     float* feat;                      // learned guess: features [n][3]
     float* gy;                        // learned guess: network output [n]
     V *mx, *mr, *mz, *mp, *mq;        // consistent-mass update [n][D]: increment, r, z, p, q = M p
