@@ -87,41 +87,21 @@ __device__ __forceinline__ float wsum(float v) {
     return v;
 }
 
-// mean of the features over the neighbours (lanes stride over the row)
-__device__ __forceinline__ void mean3(const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
-                                      const float* __restrict__ x, int64_t i, int lane, float (&m)[3], float& invdeg) {
-    const int32_t b = rp[i], e = rp[i + 1];
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-    int cnt = 0;
-    for (int32_t q = b + lane; q < e; q += 32) {
-        const int32_t j = col[q];
-        if (j != i) {
-            s0 += x[(size_t)j * 3];
-            s1 += x[(size_t)j * 3 + 1];
-            s2 += x[(size_t)j * 3 + 2];
-            ++cnt;
-        }
-    }
-    cnt = (int)wsum((float)cnt);
-    invdeg = cnt > 0 ? 1.f / (float)cnt : 0.f;
-    m[0] = wsum(s0) * invdeg;
-    m[1] = wsum(s1) * invdeg;
-    m[2] = wsum(s2) * invdeg;
-}
-
-// Sum over the neighbours j != i of v[j][lane] (rows of 32 floats): the row's
-// column indices are loaded once, 32 at a time, by the lanes of the warp and
-// broadcast with shuffles, and 8 neighbour rows are requested before any of
-// them is added, so that the warp has 8 independent 128-byte loads in flight.
-// The additions run in the row's column order (skipped entries add 0).
+// Sum over the neighbours j != i of v[j][lane] (rows of 32 floats), and their number:
+// the row's column indices are loaded once, 32 at a time, by the lanes of the warp and
+// broadcast with shuffles, and 8 neighbour rows are requested before any of them is
+// added, so that the warp has 8 independent 128-byte loads in flight.  The additions
+// run in the row's column order (skipped entries add 0).
 __device__ __forceinline__ float neighbour_sum(const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
-                                               const float* __restrict__ v, int64_t i, int lane) {
+                                               const float* __restrict__ v, int64_t i, int lane, int& degree) {
     constexpr int kU = 8;
     const int32_t b = rp[i], e = rp[i + 1];
     float s = 0.f;
+    degree = 0;
     for (int32_t c0 = b; c0 < e; c0 += 32) {
         const int cnt = min(32, (int)(e - c0));
         const int32_t mine = lane < cnt ? col[c0 + lane] : -1;
+        degree += __popc(__ballot_sync(0xffffffffu, mine >= 0 && mine != i));
         for (int t = 0; t < cnt; t += kU) {
             float x[kU];
 #pragma unroll
@@ -134,12 +114,6 @@ __device__ __forceinline__ float neighbour_sum(const int32_t* __restrict__ rp, c
         }
     }
     return s;
-}
-
-// mean of h1 over the neighbours, channel = lane
-__device__ __forceinline__ float mean_h(const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
-                                        const float* __restrict__ h, int64_t i, int lane, float invdeg) {
-    return neighbour_sum(rp, col, h, i, lane) * invdeg;
 }
 
 // ------------------------------------------------------------------ forward
@@ -155,6 +129,8 @@ __device__ __forceinline__ float gsum8(float v) {
     return v;
 }
 
+// REC: the row's inputs and neighbour means are kept as well (a.rec, for the gradients).
+template <bool REC>
 __global__ void __launch_bounds__(kBlock) k_net_l1(NetArgs a) {
     __shared__ SW s;
     load_weights(s, a.img);
@@ -193,6 +169,11 @@ __global__ void __launch_bounds__(kBlock) k_net_l1(NetArgs a) {
                 h[c4] = fmaxf(z, 0.f);
             }
             reinterpret_cast<float4*>(a.h1)[(size_t)i * (kH / 4) + lg] = make_float4(h[0], h[1], h[2], h[3]);
+            if (REC && lg == 0) {
+                float4* rec = reinterpret_cast<float4*>(a.rec) + (size_t)i * 2;
+                rec[0] = make_float4(xi[0], xi[1], xi[2], mm[0]);
+                rec[1] = make_float4(mm[1], mm[2], 0.f, 0.f);
+            }
         }
     }
 }
@@ -534,73 +515,125 @@ __global__ void __launch_bounds__(kTcThreads, 4) k_net_l2_tc(NetArgs a) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols) : "memory");
 }
 
-// layer 2 for row i: z2 (lane's channel), the neighbour mean m2 and h1_i of the lane
-__device__ __forceinline__ float layer2(const SW& s, const NetArgs& a, int64_t i, int lane, float invdeg, float& hk,
-                                        float& m2k) {
-    hk = a.h1[(size_t)i * kH + lane];
-    m2k = mean_h(a.rp, a.col, a.h1, i, lane, invdeg);
-    float z = s.c2[lane];
-#pragma unroll
-    for (int l = 0; l < kH; ++l) {
-        const float hl = __shfl_sync(0xffffffffu, hk, l);
-        const float ml = __shfl_sync(0xffffffffu, m2k, l);
-        z += s.w2aT[l * kH + lane] * hl + s.w2bT[l * kH + lane] * ml;
-    }
-    return z;
-}
-
-__device__ __forceinline__ float inv_degree(const int32_t* __restrict__ rp, const int32_t* __restrict__ col, int64_t i,
-                                            int lane) {
-    const int32_t b = rp[i], e = rp[i + 1];
-    int cnt = 0;
-    for (int32_t q = b + lane; q < e; q += 32) cnt += col[q] != i;
-    cnt = (int)wsum((float)cnt);
-    return cnt > 0 ? 1.f / (float)cnt : 0.f;
-}
-
 // ------------------------------------------------------------------ backward
+// A warp takes kBatch rows at a time, lane k owning channel k: the rows' h1, neighbour
+// mean and dz sit in shared memory, so that a weight (one load per lane) serves kBatch
+// rows and a row's values come four at a time as one broadcast load.  (One row at a
+// time, with every value broadcast by its own shuffle and every weight loaded again,
+// the shuffles and shared loads, 256 per row, were the bound: 274,625 rows, loss and
+// gradient 952 us, now 496, with the blocks' sums added by a warp per share of the
+// blocks instead of one thread over all of them.)
+constexpr int kBatch = 8;
+struct alignas(16) BatchTile {
+    float h[kBatch][kH], m[kBatch][kH], dz[kBatch][kH];
+};
+
+// acc[r] += sum_l w[l * kH + lane] * v[r][l]
+__device__ __forceinline__ void batch_product(const float* __restrict__ w, const float (*v)[kH], int lane,
+                                              float (&acc)[kBatch]) {
+#pragma unroll 2
+    for (int l = 0; l < kH; l += 4) {
+        const float w0 = w[l * kH + lane], w1 = w[(l + 1) * kH + lane], w2 = w[(l + 2) * kH + lane],
+                    w3 = w[(l + 3) * kH + lane];
+#pragma unroll
+        for (int r = 0; r < kBatch; ++r) {
+            const float4 x = *reinterpret_cast<const float4*>(&v[r][l]);
+            acc[r] += w0 * x.x;
+            acc[r] += w1 * x.y;
+            acc[r] += w2 * x.z;
+            acc[r] += w3 * x.w;
+        }
+    }
+}
+// g[l] += sum_r d[r] * v[r][l]
+__device__ __forceinline__ void batch_outer(const float (&d)[kBatch], const float (*v)[kH], float (&g)[kH]) {
+#pragma unroll
+    for (int l = 0; l < kH; l += 4)
+#pragma unroll
+        for (int r = 0; r < kBatch; ++r) {
+            const float4 x = *reinterpret_cast<const float4*>(&v[r][l]);
+            g[l] += d[r] * x.x;
+            g[l + 1] += d[r] * x.y;
+            g[l + 2] += d[r] * x.z;
+            g[l + 3] += d[r] * x.w;
+        }
+}
+
 // Layer-2 and readout gradients; stores dz2 and g = W2b^T dz2 / deg per row.
 // Block partials: [oW2a..oW2b+1024) (dW2a, dW2b), c2, w3, c3, a, and the loss.
-__global__ void __launch_bounds__(kBlock) k_net_bwd2(NetArgs a) {
-    __shared__ SW s;
-    __shared__ float red[kNetPartial];
+// Dynamic shared memory: the weights, then a tile per warp, which the block's sums
+// take over at the end.
+constexpr size_t kBwd2Smem = sizeof(SW) + kWarps * sizeof(BatchTile);
+static_assert(kWarps * sizeof(BatchTile) >= kNetPartial * sizeof(float), "the block's sums fit in the tiles");
+__global__ void __launch_bounds__(kBlock, 2) k_net_bwd2(NetArgs a) {
+    extern __shared__ __align__(16) unsigned char bw_dsm[];
+    SW& s = *reinterpret_cast<SW*>(bw_dsm);
     load_weights(s, a.img);
-    for (int q = threadIdx.x; q < kNetPartial; q += blockDim.x) red[q] = 0.f;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    BatchTile& t = reinterpret_cast<BatchTile*>(bw_dsm + sizeof(SW))[wib];
     const int64_t w0 = ((int64_t)blockIdx.x * kBlock + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * kBlock) >> 5;
     float gw2a[kH], gw2b[kH];
 #pragma unroll
     for (int l = 0; l < kH; ++l) gw2a[l] = gw2b[l] = 0.f;
     float gc2 = 0.f, gw3 = 0.f, gc3 = 0.f, ga0 = 0.f, ga1 = 0.f, loss = 0.f;
     const float scale = 2.f / (float)a.n;
-    for (int64_t i = w0; i < a.n; i += nw) {
-        const float invdeg = inv_degree(a.rp, a.col, i, lane);
-        float hk, m2k;
-        const float z = layer2(s, a, i, lane, invdeg, hk, m2k);
-        const float h2 = fmaxf(z, 0.f);
-        const float* xi = a.x + (size_t)i * 3;
-        const float y = wsum(s.w3[lane] * h2) + s.c3 + s.a0 * xi[1] + s.a1 * xi[2];
-        const float r = y - a.t[i];
-        const float dy = scale * r;
-        loss += lane == 0 ? r * r : 0.f;
-        gc3 += lane == 0 ? dy : 0.f;
-        ga0 += lane == 0 ? dy * xi[1] : 0.f;
-        ga1 += lane == 0 ? dy * xi[2] : 0.f;
-        gw3 += dy * h2;
-        const float dz = z > 0.f ? dy * s.w3[lane] : 0.f;
-        gc2 += dz;
+    for (int64_t i0 = w0 * kBatch; i0 < a.n; i0 += nw * kBatch) {
+        const int rows = (int)min((int64_t)kBatch, a.n - i0);
+        float invdeg[kBatch];
 #pragma unroll
-        for (int l = 0; l < kH; ++l) {
-            gw2a[l] += dz * __shfl_sync(0xffffffffu, hk, l);
-            gw2b[l] += dz * __shfl_sync(0xffffffffu, m2k, l);
+        for (int r = 0; r < kBatch; ++r) {
+            float h = 0.f, m = 0.f;
+            int deg = 0;
+            if (r < rows) {
+                h = a.h1[(size_t)(i0 + r) * kH + lane];
+                m = neighbour_sum(a.rp, a.col, a.h1, i0 + r, lane, deg);
+            }
+            invdeg[r] = deg > 0 ? 1.f / (float)deg : 0.f;
+            t.h[r][lane] = h;
+            t.m[r][lane] = m * invdeg[r];
         }
-        a.dz2[(size_t)i * kH + lane] = dz;
-        float g = 0.f;
+        __syncwarp();
+        float z[kBatch];
 #pragma unroll
-        for (int l = 0; l < kH; ++l) g += s.w2b[l * kH + lane] * __shfl_sync(0xffffffffu, dz, l);
-        a.g[(size_t)i * kH + lane] = g * invdeg;
+        for (int r = 0; r < kBatch; ++r) z[r] = s.c2[lane];
+        batch_product(s.w2aT, t.h, lane, z);
+        batch_product(s.w2bT, t.m, lane, z);
+        float dz[kBatch];
+#pragma unroll
+        for (int r = 0; r < kBatch; ++r) {
+            dz[r] = 0.f;
+            if (r < rows) {
+                const float h2 = fmaxf(z[r], 0.f);
+                const float* xi = a.x + (size_t)(i0 + r) * 3;
+                const float y = wsum(s.w3[lane] * h2) + s.c3 + s.a0 * xi[1] + s.a1 * xi[2];
+                const float res = y - a.t[i0 + r];
+                const float dy = scale * res;
+                loss += lane == 0 ? res * res : 0.f;
+                gc3 += lane == 0 ? dy : 0.f;
+                ga0 += lane == 0 ? dy * xi[1] : 0.f;
+                ga1 += lane == 0 ? dy * xi[2] : 0.f;
+                gw3 += dy * h2;
+                dz[r] = z[r] > 0.f ? dy * s.w3[lane] : 0.f;
+                gc2 += dz[r];
+                a.dz2[(size_t)(i0 + r) * kH + lane] = dz[r];
+            }
+            t.dz[r][lane] = dz[r];
+        }
+        __syncwarp();
+        batch_outer(dz, t.h, gw2a);
+        batch_outer(dz, t.m, gw2b);
+        float g[kBatch] = {};
+        batch_product(s.w2b, t.dz, lane, g);
+#pragma unroll
+        for (int r = 0; r < kBatch; ++r)
+            if (r < rows) a.g[(size_t)(i0 + r) * kH + lane] = g[r] * invdeg[r];
+        __syncwarp();
     }
     // per-block sums in warp order (deterministic)
+    float* red = reinterpret_cast<float*>(bw_dsm + sizeof(SW));
+    __syncthreads();
+    for (int q = threadIdx.x; q < kNetPartial; q += blockDim.x) red[q] = 0.f;
+    __syncthreads();
     for (int w = 0; w < kWarps; ++w) {
         if (wib == w) {
 #pragma unroll
@@ -623,34 +656,44 @@ __global__ void __launch_bounds__(kBlock) k_net_bwd2(NetArgs a) {
     for (int q = threadIdx.x; q < kNetPartial; q += blockDim.x) out[oW2a + q] = red[q];
 }
 
-// Layer-1 gradients: dh1 = W2a^T dz2 + sum_{j in N(i)} g_j, dz1 = dh1 [z1 > 0].
+// Layer-1 gradients: dh1 = W2a^T dz2 + sum_{j in N(i)} g_j, dz1 = dh1 [z1 > 0]; the
+// row's inputs and neighbour means come from the record that layer 1 kept.
 __global__ void __launch_bounds__(kBlock) k_net_bwd1(NetArgs a) {
     __shared__ SW s;
     __shared__ float red[oW2a];
+    __shared__ __align__(16) float tile[kWarps][kBatch][kH];
     load_weights(s, a.img);
     for (int q = threadIdx.x; q < oW2a; q += blockDim.x) red[q] = 0.f;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int64_t w0 = ((int64_t)blockIdx.x * kBlock + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * kBlock) >> 5;
     float gw1a[3] = {0.f, 0.f, 0.f}, gw1b[3] = {0.f, 0.f, 0.f}, gc1 = 0.f;
-    for (int64_t i = w0; i < a.n; i += nw) {
-        float m[3], invdeg;
-        mean3(a.rp, a.col, a.x, i, lane, m, invdeg);
-        const float* xi = a.x + (size_t)i * 3;
-        float z = s.c1[lane];
+    for (int64_t i0 = w0 * kBatch; i0 < a.n; i0 += nw * kBatch) {
+        const int rows = (int)min((int64_t)kBatch, a.n - i0);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) z += s.w1a[lane * 3 + c] * xi[c] + s.w1b[lane * 3 + c] * m[c];
-        const float dzi = a.dz2[(size_t)i * kH + lane];
-        float dh = 0.f;
+        for (int r = 0; r < kBatch; ++r) tile[wib][r][lane] = r < rows ? a.dz2[(size_t)(i0 + r) * kH + lane] : 0.f;
+        __syncwarp();
+        float dh[kBatch] = {};
+        batch_product(s.w2a, tile[wib], lane, dh);
 #pragma unroll
-        for (int l = 0; l < kH; ++l) dh += s.w2a[l * kH + lane] * __shfl_sync(0xffffffffu, dzi, l);
-        dh += neighbour_sum(a.rp, a.col, a.g, i, lane);
-        const float dz = z > 0.f ? dh : 0.f;
-        gc1 += dz;
+        for (int r = 0; r < kBatch; ++r) {
+            if (r >= rows) break;
+            int deg;
+            const float dr = dh[r] + neighbour_sum(a.rp, a.col, a.g, i0 + r, lane, deg);
+            const float4 p = reinterpret_cast<const float4*>(a.rec)[(size_t)(i0 + r) * 2];
+            const float4 q = reinterpret_cast<const float4*>(a.rec)[(size_t)(i0 + r) * 2 + 1];
+            const float xi[3] = {p.x, p.y, p.z}, m[3] = {p.w, q.x, q.y};
+            float z = s.c1[lane];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            gw1a[c] += dz * xi[c];
-            gw1b[c] += dz * m[c];
+            for (int c = 0; c < 3; ++c) z += s.w1a[lane * 3 + c] * xi[c] + s.w1b[lane * 3 + c] * m[c];
+            const float dz = z > 0.f ? dr : 0.f;
+            gc1 += dz;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                gw1a[c] += dz * xi[c];
+                gw1b[c] += dz * m[c];
+            }
         }
+        __syncwarp();
     }
     for (int w = 0; w < kWarps; ++w) {
         if (wib == w) {
@@ -667,14 +710,25 @@ __global__ void __launch_bounds__(kBlock) k_net_bwd1(NetArgs a) {
     for (int q = threadIdx.x; q < oW2a; q += blockDim.x) out[q] = red[q];
 }
 
-// grad[p] = sum over blocks (in block order) of the partials; loss likewise.
-__global__ void k_net_reduce(const float* __restrict__ partial, int blocks, float* __restrict__ grad,
-                             float* __restrict__ loss, int n) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p > kNetParams) return;
+// grad[p] = sum over blocks of the partials (each warp a contiguous share of the
+// blocks in order, then the warps in order); loss likewise.  32 parameters per block.
+__global__ void __launch_bounds__(kBlock) k_net_reduce(const float* __restrict__ partial, int blocks2, int blocks1,
+                                                       float* __restrict__ grad, float* __restrict__ loss, int n) {
+    __shared__ float sh[kWarps][32];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int p = blockIdx.x * 32 + lane;
     const int col = p < kNetParams ? p : oW2a + kNetPartial - 1;
+    const int blocks = p < oW2a ? blocks1 : blocks2;
+    const int per = (blocks + kWarps - 1) / kWarps, b1 = min(blocks, (wib + 1) * per);
     float acc = 0.f;
-    for (int b = 0; b < blocks; ++b) acc += partial[(size_t)b * kNetPartialStride + col];
+    if (p <= kNetParams) {
+#pragma unroll 8
+        for (int b = wib * per; b < b1; ++b) acc += partial[(size_t)b * kNetPartialStride + col];
+    }
+    sh[wib][lane] = acc;
+    __syncthreads();
+    if (wib != 0 || p > kNetParams) return;
+    for (int w = 1; w < kWarps; ++w) acc += sh[w][lane];
     if (p < kNetParams) grad[p] = acc;
     else *loss = acc / (float)n;
 }
@@ -700,9 +754,13 @@ __global__ void k_net_to_bf16(const float* __restrict__ p32, __nv_bfloat16* __re
     if (q < kNetParams) p16[q] = __float2bfloat16_rn(p32[q]);
 }
 
-int net_grid(int64_t rows) {
-    const int64_t want = (rows + kWarps - 1) / kWarps;
-    return (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)num_sms() * 8));
+// one resident wave of a gradient kernel, kBatch rows per warp at a time
+template <class K>
+int net_grid(K kernel, size_t smem, int64_t rows) {
+    int per_sm = 0;
+    OASIS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBlock, smem));
+    const int64_t want = (rows + kWarps * kBatch - 1) / (kWarps * kBatch);
+    return (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)num_sms() * std::max(1, per_sm)));
 }
 }  // namespace
 
@@ -723,7 +781,9 @@ Net* net_create(const Mesh& m) {
     N->h1.alloc((size_t)m.n * kH);
     N->dz2.alloc((size_t)m.n * kH);
     N->g.alloc((size_t)m.n * kH);
-    N->grid = net_grid(m.n);
+    OASIS_CUDA(cudaFuncSetAttribute(k_net_bwd2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBwd2Smem));
+    N->grid = net_grid(k_net_bwd2, kBwd2Smem, m.n);
+    N->grid1 = net_grid(k_net_bwd1, 0, m.n);
     N->img.alloc(sizeof(SW) / sizeof(float));
     k_net_image<<<4, 256>>>(N->p16.p, N->img.p);
     N->bop.alloc((size_t)kH * kTcK);
@@ -759,11 +819,11 @@ Net* net_create(const Mesh& m) {
     const int64_t tc_tiles = (m.n + kTcRows - 1) / kTcRows;
     N->grid_tc = (int)std::max<int64_t>(1, std::min<int64_t>(tc_tiles, (int64_t)per_sm_tc * num_sms()));
     int per_sm = 0;
-    OASIS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_net_l1, kBlock, 0));
+    OASIS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_net_l1<false>, kBlock, 0));
     const int64_t groups = (m.n + kRowsPerWarp - 1) / kRowsPerWarp;
     N->grid_fwd = (int)std::max<int64_t>(
         1, std::min<int64_t>((groups + kWarps - 1) / kWarps, (int64_t)std::max(per_sm, 1) * num_sms()));
-    N->partial.alloc((size_t)N->grid * kNetPartialStride);
+    N->partial.alloc((size_t)std::max(N->grid, N->grid1) * kNetPartialStride);
     OASIS_CUDA(cudaDeviceSynchronize());
     return N.release();
 }
@@ -791,7 +851,7 @@ NetArgs net_args(Net& N, const float* x, float* y, const float* t) {
 void net_forward(Net& N, const float* x, float* y, cudaStream_t s) {
     const NetArgs a = net_args(N, x, y, nullptr);
     if (kInferStoredH1) {
-        k_net_l1<<<N.grid_fwd, kBlock, 0, s>>>(a);
+        k_net_l1<false><<<N.grid_fwd, kBlock, 0, s>>>(a);
         k_net_l2_tc<true><<<N.grid_tc, kTcThreads, kTcSmem, s>>>(a);
     } else {
         k_net_rec<<<N.grid_fwd, kBlock, 0, s>>>(a);
@@ -812,11 +872,11 @@ void net_check(Net& N, cudaStream_t s) {
 
 void net_backward(Net& N, const float* x, const float* t, float* grad, float* loss, cudaStream_t s) {
     const NetArgs a = net_args(N, x, nullptr, t);
-    k_net_l1<<<N.grid_fwd, kBlock, 0, s>>>(a);
-    k_net_bwd2<<<N.grid, kBlock, 0, s>>>(a);
-    k_net_bwd1<<<N.grid, kBlock, 0, s>>>(a);
-    k_net_reduce<<<(kNetParams + 1 + 255) / 256, 256, 0, s>>>(N.partial.p, N.grid, grad ? grad : N.grad.p,
-                                                             loss ? loss : N.loss.p, (int)N.n);
+    k_net_l1<true><<<N.grid_fwd, kBlock, 0, s>>>(a);
+    k_net_bwd2<<<N.grid, kBlock, kBwd2Smem, s>>>(a);
+    k_net_bwd1<<<N.grid1, kBlock, 0, s>>>(a);
+    k_net_reduce<<<(kNetParams + 1 + 31) / 32, kBlock, 0, s>>>(N.partial.p, N.grid, N.grid1, grad ? grad : N.grad.p,
+                                                               loss ? loss : N.loss.p, (int)N.n);
     OASIS_CUDA(cudaGetLastError());
 }
 

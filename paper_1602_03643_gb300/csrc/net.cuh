@@ -31,7 +31,7 @@ struct NetArgs {
 struct Net {
     const Mesh* m = nullptr;
     int64_t n = 0;
-    int grid = 1;
+    int grid = 1, grid1 = 1;
     DBuf<float> p32, mom, var, grad, loss;
     DBuf<__nv_bfloat16> p16;
     DBuf<float> img;     // bfloat16 weights widened to float, in shared-memory layout
