@@ -280,8 +280,8 @@ int oasis_mesh_get_pattern(const oasis_mesh* mesh, int32_t* row_ptr, int32_t* co
 int oasis_mesh_get_matrix(const oasis_mesh* mesh, int32_t which, double* values);
 
 /* y = Mat x on device vectors of length n_dofs (float64, internal dof order), Mat
- * one of the constant matrices, with `lanes` lanes per row (0 = 16).  For
- * kernel-level tests and bandwidth measurements. */
+ * one of the constant matrices, with `lanes` lanes per row (4, 8, 16 or 32; 0 = the
+ * library's choice).  For kernel-level tests and bandwidth measurements. */
 int oasis_spmv_f64(const oasis_mesh* mesh, int32_t which, const double* x, double* y,
                    int32_t lanes, void* stream);
 /* Same in float32 values and vectors (the values are the float32 copy of the matrix). */
@@ -290,9 +290,9 @@ int oasis_spmv_f32(const oasis_mesh* mesh, int32_t which, const float* x, float*
 
 /* y = Mat x and *xy = x . y in float64 (for K this is the energy product p . K p
  * of the CG iteration, Sec. 6 solvers), on device vectors of length n_dofs; xy
- * is one double in device memory.  Row tiles of 256 rows, one partial sum per
- * tile in scratch owned by the mesh (allocated by oasis_assemble_constant), and
- * a deterministic final sum in tile order.  Calls on one mesh must not overlap
+ * is one double in device memory.  One partial sum per block in scratch owned by
+ * the mesh (allocated by oasis_assemble_constant), and a deterministic final sum
+ * in block order.  Calls on one mesh must not overlap
  * on the GPU (they share that scratch). */
 int oasis_spmv_dot_f64(const oasis_mesh* mesh, int32_t which, const double* x, double* y, double* xy,
                        void* stream);
@@ -303,7 +303,7 @@ int oasis_spmv_dot_f64(const oasis_mesh* mesh, int32_t which, const double* x, d
  * allocates nothing.  The paper has no counterpart; it is a deployment variant.
  *   - Its reduction scratch is a file-scope __device__ array of 516 KiB that
  *     every GPU loading the library holds until process exit; it limits n_dofs
- *     to 16,777,216 (65,536 tiles of 256 rows).  Larger meshes: OASIS_EINVAL.
+ *     to 16,777,216 (one partial sum per 256 rows).  Larger meshes: OASIS_EINVAL.
  *   - The first call on a device resolves the array's device address
  *     (cudaGetSymbolAddress) with that device current; make that first call
  *     before any stream capture.

@@ -1,8 +1,6 @@
 // Smoothed-aggregation AMG for the pressure operator: host setup (once per
 // mesh, from the assembled float64 K) and the V(1,1) cycle kernels.
 #include <algorithm>
-#include <map>
-#include <mutex>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -1028,24 +1026,6 @@ __global__ void __launch_bounds__(kDenseBlock) k_amg_dense(int64_t n, int64_t ld
         if (threadIdx.x == 0) x[i] = (sh[0] + sh[1]) + (sh[2] + sh[3]);
         __syncthreads();
     }
-}
-
-// Blocks of `fn` (kBlock threads, no dynamic shared memory) resident on one SM
-// of the current device, from the occupancy calculator, cached per device and
-// kernel: grids of grid-stride kernels stay within one wave.
-int resident_blocks(const void* fn) {
-    static std::mutex mu;
-    static std::map<std::pair<int, const void*>, int> cache;
-    int dev = 0;
-    OASIS_CUDA(cudaGetDevice(&dev));
-    std::lock_guard<std::mutex> lock(mu);
-    auto it = cache.find({dev, fn});
-    if (it != cache.end()) return it->second;
-    int per_sm = 0;
-    OASIS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlock, 0));
-    per_sm = std::max(1, per_sm);
-    cache[{dev, fn}] = per_sm;
-    return per_sm;
 }
 
 // finest-level sweeps: one warp per slice pair at a time, one resident wave

@@ -441,7 +441,7 @@ int oasis_spmv_f64(const oasis_mesh* mesh, int32_t which, const double* x, doubl
         const Mesh* m = reinterpret_cast<const Mesh*>(mesh);
         OASIS_CHECK(m && x && y, OASIS_EINVAL, "null pointer");
         OASIS_CHECK(m->assembled, OASIS_EINVAL, "mesh not assembled");
-        spmv_f64(*m, (const double*)const_matrix(m, which, false), x, y, lanes ? lanes : 16, as_stream(stream));
+        spmv_f64(*m, (const double*)const_matrix(m, which, false), x, y, lanes, as_stream(stream));
     });
 }
 
@@ -450,7 +450,7 @@ int oasis_spmv_f32(const oasis_mesh* mesh, int32_t which, const float* x, float*
         const Mesh* m = reinterpret_cast<const Mesh*>(mesh);
         OASIS_CHECK(m && x && y, OASIS_EINVAL, "null pointer");
         OASIS_CHECK(m->assembled, OASIS_EINVAL, "mesh not assembled");
-        spmv_f32(*m, (const float*)const_matrix(m, which, true), x, y, lanes ? lanes : 16, as_stream(stream));
+        spmv_f32(*m, (const float*)const_matrix(m, which, true), x, y, lanes, as_stream(stream));
     });
 }
 

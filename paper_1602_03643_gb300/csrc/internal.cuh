@@ -129,7 +129,7 @@ struct Mesh {
     DBuf<float> K32s;
     DBuf<double> K64s;
     DBuf<float2> Kffs;
-    DBuf<double> red_partial;                  // one partial sum per 256-row tile
+    DBuf<double> red_partial;                  // room for one partial sum per 256 rows
     DBuf<uint32_t> red_ticket;
     DBuf<int32_t> err;                         // device error flag for setup kernels
     bool assembled = false;
@@ -168,11 +168,15 @@ struct Solver;
 // Kernels and launchers (step.cu)
 void spmv_f64(const Mesh& m, const double* vals, const double* x, double* y, int lanes, cudaStream_t s);
 void spmv_f32(const Mesh& m, const float* vals, const float* x, float* y, int lanes, cudaStream_t s);
-void spmv_dot_f64(const Mesh& m, const double* vals, const double* x, double* y, double* xy, double* tile_partial,
+void spmv_dot_f64(const Mesh& m, const double* vals, const double* x, double* y, double* xy, double* partial,
                   uint32_t* ticket, cudaStream_t s);
 void noalloc_scratch(double** partial, uint32_t** ticket);
 int64_t noalloc_max_rows();
 
 int num_sms();
+// Blocks of `fn` (kBlock threads, no dynamic shared memory) resident on one SM of the
+// current device, from the occupancy calculator, cached per device and kernel: grids of
+// grid-stride kernels stay within one wave.
+int resident_blocks(const void* fn);
 
 }  // namespace oasis

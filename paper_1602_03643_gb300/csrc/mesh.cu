@@ -3,6 +3,7 @@
 // stand-alone SpMV kernels.
 #include <algorithm>
 #include <cmath>
+#include <map>
 #include <numeric>
 #include <mutex>
 #include <thread>
@@ -20,6 +21,21 @@ int num_sms() {
         OASIS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     }
     return sms;
+}
+
+int resident_blocks(const void* fn) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void*>, int> cache;
+    int dev = 0;
+    OASIS_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = cache.find({dev, fn});
+    if (it != cache.end()) return it->second;
+    int per_sm = 0;
+    OASIS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlock, 0));
+    per_sm = std::max(1, per_sm);
+    cache[{dev, fn}] = per_sm;
+    return per_sm;
 }
 
 // ------------------------------------------------------------------ host build
@@ -543,8 +559,114 @@ __global__ void __launch_bounds__(kBlock) k_spmv(int64_t n, const int32_t* __res
     }
 }
 
+// The library's own choice: G lanes per row and U rows in flight per lane group (row
+// pointers, then one entry of every row per round), the grid one resident wave; columns
+// as the pattern's 16-bit offsets from the row, modulo n, where it has them (C16: 6
+// bytes per float32 entry instead of 8, 10 per float64 entry instead of 12).  DOT: x . y
+// as well, one partial sum per block, added in block order by the block that takes the
+// last ticket (`ticket` must be zero at launch; it is left zero).
+// Bound by the dependent loads row pointer -> column -> operand, so rows in flight
+// count.  1,030,200 rows, 15.2 M entries in reverse Cuthill-McKee order, one product
+// each with M in float64, K in float32 and K in float64 with the dot: 393 us with 16
+// lanes per row and one row at a time (DOT: 256-row tiles through shared memory), 160
+// with this form; the bytes alone take 72 at the copy rate.
+template <class V, int G, int U, bool C16, bool DOT>
+__global__ void __launch_bounds__(kBlock) k_spmv_rows(int64_t n, const int32_t* __restrict__ rp,
+                                                      const int32_t* __restrict__ col,
+                                                      const int16_t* __restrict__ dcol, const V* __restrict__ val,
+                                                      const V* __restrict__ x, V* __restrict__ y,
+                                                      double* __restrict__ partial, uint32_t* ticket,
+                                                      double* __restrict__ xy) {
+    constexpr int RPW = 32 / G;
+    const int lane = threadIdx.x & 31, lg = lane & (G - 1), grp = lane / G;
+    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const uint32_t n32 = (uint32_t)n;
+    double dot[1] = {0.0};
+    for (int64_t base = w0 * RPW * U; base < n; base += nw * RPW * U) {
+        uint32_t i[U];
+        int32_t q[U], e[U];
+        V acc[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            i[u] = (uint32_t)(base + u * RPW + grp);
+            const bool ok = i[u] < n32;
+            q[u] = ok ? rp[i[u]] + lg : 0;
+            e[u] = ok ? rp[i[u] + 1] : 0;
+            acc[u] = 0;
+        }
+        bool more = false;
+#pragma unroll
+        for (int u = 0; u < U; ++u) more |= q[u] < e[u];
+        while (more) {
+            uint32_t j[U];
+            V av[U], g[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const bool has = q[u] < e[u];
+                uint32_t jc = 0;
+                if constexpr (C16) {
+                    // row + offset, wrapped once into [0, n)
+                    int32_t jj = (int32_t)i[u] + (int32_t)(has ? dcol[q[u]] : (int16_t)0);
+                    jj = jj < 0 ? jj + (int32_t)n32 : jj;
+                    jc = (uint32_t)jj >= n32 ? (uint32_t)jj - n32 : (uint32_t)jj;
+                } else {
+                    jc = has ? (uint32_t)col[q[u]] : 0u;
+                }
+                j[u] = has ? jc : 0u;
+                av[u] = has ? val[q[u]] : V(0);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) g[u] = x[j[u]];
+            more = false;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (q[u] < e[u]) {
+                    acc[u] += av[u] * g[u];
+                    q[u] += G;
+                }
+                more |= q[u] < e[u];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const V sum = group_sum<G>(acc[u]);
+            if (i[u] < n32 && lg == 0) {
+                y[i[u]] = sum;
+                if constexpr (DOT) dot[0] += x[i[u]] * sum;
+            }
+        }
+    }
+    if constexpr (DOT) {
+        if (grid_sum<1>(dot, partial, ticket) && threadIdx.x == 0) *xy = dot[0];
+    }
+}
+
+// One resident wave of a grid-stride kernel with `rows` rows per block at a time.
+static int wave_grid(const void* fn, int64_t n, int64_t rows) {
+    const int64_t want = (n + rows - 1) / rows;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)num_sms() * resident_blocks(fn)));
+}
+
+template <class V, bool DOT>
+static void spmv_rows(const Mesh& m, const V* vals, const V* x, V* y, double* partial, uint32_t* ticket, double* xy,
+                      cudaStream_t s) {
+    constexpr int G = 2, U = 4;
+    auto run = [&](auto fn) {
+        fn<<<wave_grid((const void*)fn, m.n, (int64_t)kBlock / G * U), kBlock, 0, s>>>(
+            m.n, m.row_ptr.p, m.col.p, m.csr_dcol.p, vals, x, y, partial, ticket, xy);
+    };
+    if (m.csr_dcol.p) run(k_spmv_rows<V, G, U, true, DOT>);
+    else run(k_spmv_rows<V, G, U, false, DOT>);
+    OASIS_CUDA(cudaGetLastError());
+}
+
 template <class V>
 static void spmv_launch(const Mesh& m, const V* vals, const V* x, V* y, int lanes, cudaStream_t s) {
+    if (lanes == 0) {
+        spmv_rows<V, false>(m, vals, x, y, nullptr, nullptr, nullptr, s);
+        return;
+    }
     const int rows_per_block = kBlock / lanes;
     const int g = grid_for(m.n, rows_per_block);
     switch (lanes) {
@@ -557,88 +679,12 @@ static void spmv_launch(const Mesh& m, const V* vals, const V* x, V* y, int lane
     OASIS_CUDA(cudaGetLastError());
 }
 
-// y = Mat x and x . y in float64 with 256-row tiles: an entry-parallel product
-// phase into shared memory, a thread-per-row sum, one partial sum per tile in
-// `tile_partial`, and a deterministic final sum (in tile order) by the block
-// that takes the last ticket.  `ticket` must be zero at launch; it is left zero.
-__global__ void __launch_bounds__(kBlock) k_spmv_dot_tiles(int64_t n, const int32_t* __restrict__ rp,
-                                                           const int32_t* __restrict__ col,
-                                                           const double* __restrict__ val,
-                                                           const double* __restrict__ x, double* __restrict__ y,
-                                                           double* __restrict__ tile_partial, uint32_t* ticket,
-                                                           double* __restrict__ xy) {
-    extern __shared__ __align__(16) unsigned char dsm[];
-    double* s_prod = reinterpret_cast<double*>(dsm);
-    __shared__ int32_t s_rp[kBlock + 1];
-    const int64_t ntiles = (n + kBlock - 1) / kBlock;
-    const int r = threadIdx.x;
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int64_t r0 = tile * kBlock;
-        const int nr = (int)min((int64_t)kBlock, n - r0);
-        for (int k = r; k <= nr; k += blockDim.x) s_rp[k] = rp[r0 + k];
-        __syncthreads();
-        const int32_t e0 = s_rp[0], e1 = s_rp[nr];
-        for (int32_t e = e0 + r; e < e1; e += kBlock) s_prod[e - e0] = val[e] * x[col[e]];
-        __syncthreads();
-        double v[1] = {0.0};
-        if (r < nr) {
-            double acc = 0.0;
-            for (int32_t q = s_rp[r] - e0; q < s_rp[r + 1] - e0; ++q) acc += s_prod[q];
-            y[r0 + r] = acc;
-            v[0] = x[r0 + r] * acc;
-        }
-        block_sum<1>(v);
-        if (r == 0) tile_partial[tile] = v[0];
-        __syncthreads();
-    }
-    __shared__ bool last;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    double s[1] = {0.0};
-    for (int64_t t = threadIdx.x; t < ntiles; t += blockDim.x) s[0] += __ldcg(&tile_partial[t]);
-    block_sum<1>(s);
-    if (threadIdx.x == 0) {
-        *xy = s[0];
-        *ticket = 0u;
-    }
-}
-
-void spmv_dot_f64(const Mesh& m, const double* vals, const double* x, double* y, double* xy, double* tile_partial,
+// y = Mat x and x . y in float64; `partial` holds one double per block (at least one
+// per 256 rows, and never more blocks than that).
+void spmv_dot_f64(const Mesh& m, const double* vals, const double* x, double* y, double* xy, double* partial,
                   uint32_t* ticket, cudaStream_t s) {
-    const int64_t ntiles = (m.n + kBlock - 1) / kBlock;
-    const size_t smem = (size_t)std::max(1, m.tile_cap) * sizeof(double);
-    // The opt-in dynamic shared-memory size is a per-device attribute of the
-    // kernel: it is set once per device (with that device current) and cached
-    // under a lock, so concurrent first calls and later devices are covered.
-    static std::mutex mu;
-    static int rooms[256] = {0};
-    int dev = 0;
-    OASIS_CUDA(cudaGetDevice(&dev));
-    OASIS_CHECK(dev >= 0 && dev < 256, OASIS_EINVAL, "device ordinal out of range");
-    int room = 0;
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        if (!rooms[dev]) {
-            int optin = 0;
-            OASIS_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-            cudaFuncAttributes fa{};
-            OASIS_CUDA(cudaFuncGetAttributes(&fa, k_spmv_dot_tiles));
-            const int r = optin - (int)fa.sharedSizeBytes;
-            OASIS_CUDA(cudaFuncSetAttribute(k_spmv_dot_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, r));
-            rooms[dev] = r;
-        }
-        room = rooms[dev];
-    }
-    OASIS_CHECK(smem <= (size_t)room, OASIS_EINVAL, "a row tile needs more shared memory than the device offers");
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(ntiles, (int64_t)num_sms() * 4));
     OASIS_CUDA(cudaMemsetAsync(ticket, 0, sizeof(uint32_t), s));
-    k_spmv_dot_tiles<<<grid, kBlock, smem, s>>>(m.n, m.row_ptr.p, m.col.p, vals, x, y, tile_partial, ticket, xy);
-    OASIS_CUDA(cudaGetLastError());
+    spmv_rows<double, true>(m, vals, x, y, partial, ticket, xy, s);
 }
 
 // ------------------------------------------------------------------ no-alloc scratch
@@ -646,7 +692,7 @@ void spmv_dot_f64(const Mesh& m, const double* vals, const double* x, double* y,
 // allocate device memory (code running under a caller-owned memory pool or
 // inside an allocator, or on a device that is already full).  Every GPU that
 // loads the library holds these arrays until the process exits (516 KiB).
-// One partial sum per 256-row tile: at most 65,536 tiles, i.e. 16,777,216 rows.
+// Room for one partial sum per 256 rows: at most 65,536, i.e. 16,777,216 rows.
 constexpr int64_t kNoAllocMaxTiles = 65536;
 static __device__ __align__(256) double g_noalloc_partial[kNoAllocMaxTiles];
 static __device__ __align__(256) uint32_t g_noalloc_ticket[64];
