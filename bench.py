@@ -83,6 +83,18 @@ MEASURED_TRAFFIC = {("stress128_rcm", "pcg_spmv@sell"): (215.0e6, _S112),
                     ("stress128_rcm", "bicg_spmm@rows16"): (263.6e6, _S112)}
 
 
+# Sizes up to which the library runs a linear solve as one resident launch in the
+# captured step (kResidentRows, kResidentAmgEntries), and below which the V-cycle's
+# levels share one launch (kTailRows)
+RESIDENT_ROWS, RESIDENT_AMG_ENTRIES, TAIL_ROWS = 650_000, 1_900_000, 40_000
+
+
+def amg_tail(amg):
+    """First level of the V-cycle's shared launch (the number of operator levels if none)."""
+    ops = amg["levels"] - 1
+    return next((l for l in range(1, ops) if amg["rows"][l] <= TAIL_ROWS), ops)
+
+
 def family_bytes(pb, nnz, args, tuning, amg):
     """Algorithmic bytes per launch of every timed kernel family (float32 values,
     int32 indices unless stated; N dofs, Z pattern entries, T cells, D dims; each
@@ -103,6 +115,9 @@ def family_bytes(pb, nnz, args, tuning, amg):
       amg_coarse   coarser-level sweeps (bfloat16 values) and the dense coarsest product,
                    averaged over their 2(L-2)+1 launches: per sweep 6 nnz_l + 20 n_l (CSR)
                    or 4 nnz_l + 16.5 n_l (pair-packed); dense 4 nc ld + 8 nc
+                   With amg["tail"] the levels from there on share one launch: their
+                   transfers count in amg_coarse, over 2 tail transfer launches and
+                   2(tail-1)+1 coarse ones
       bicg_vec     BiCGStab vector kernels, averaged over dir (64 N), s (52 N), and
                    the solution/residual update with its dots (96 N), for D = 3
       assemble     convecting velocity per dof (u^{n-1}, u^{n-2} read, ubar written: 60 N),
@@ -112,7 +127,8 @@ def family_bytes(pb, nnz, args, tuning, amg):
                    solve's (A + columns 8 Z; r0, Delta gathered, r, rh, p, v, dl: 112 N)
                    and the pressure's (K as float-float + columns 12 Z; 56 N)
       pcg_update   multigrid CG vector update: u, w, p, s, increment, r read, p, s,
-                   increment, r written (40 N)
+                   increment, r written (40 N; the diagonal inverse read and the cycle's
+                   first sweep written beside them, 8 N, are not counted)
     Returns {family: (kernel, bytes per launch, formula)}."""
     N, Z, T, D = pb.mesh.n_dofs, nnz, pb.mesh.n_cells, pb.mesh.dim
     n_slices = (N + 31) // 32
@@ -130,6 +146,7 @@ def family_bytes(pb, nnz, args, tuning, amg):
         rows, nz, pn = amg["rows"], amg["nnz"], amg["p_nnz"]
         packed = amg.get("packed") or [0] * len(pn)
         L = amg["levels"]
+        tail = amg.get("tail", L - 1)
         if pn:
             # restriction: entries, R's row pointers (CSR) or slice headers (packed), the
             # fine residual gathered, the coarse vector written; prolongation: entries,
@@ -145,24 +162,26 @@ def family_bytes(pb, nnz, args, tuning, amg):
                 eb = 6 if packed[l] & 32 else 4
                 return (eb * pn[l] + 8.5 * rows[l] + 4 * rows[l + 1] if packed[l] & 4
                         else 6 * pn[l] + 12 * rows[l] + 4 * rows[l + 1])
-            tb = sum(restrict_b(l) + prolong_b(l) for l in range(len(pn)))
+            tb = sum(restrict_b(l) + prolong_b(l) for l in range(tail))
+            tail_b = sum(restrict_b(l) + prolong_b(l) for l in range(tail, len(pn)))
             out["amg_transfer"] = ("k_amg_restrict / k_amg_prolong (CSR) and k_amg_sellp (pair-packed SELL-32), "
-                                   "bfloat16 values, every level", tb / (2 * len(pn)),
+                                   "bfloat16 values, every level before the shared launch", tb / (2 * tail),
                                    "per V-cycle sum_l: restriction 6 nnz(P_l) + 4 n_l + 8 n_(l+1) (CSR) or "
                                    "4 nnz(P_l) + 4 n_l + 4.5 n_(l+1) (packed); prolongation 6 nnz(P_l) + 12 n_l "
-                                   "+ 4 n_(l+1) or 4 nnz(P_l) + 8.5 n_l + 4 n_(l+1); over 2(L-1) launches")
+                                   "+ 4 n_(l+1) or 4 nnz(P_l) + 8.5 n_l + 4 n_(l+1); over 2 launches per level")
         nc = rows[L - 1]
         ld = (nc + 3) // 4 * 4
 
         def sweep_b(l):
             eb = 6 if packed[l] & 8 else 4
             return eb * nz[l] + 16.5 * rows[l] if packed[l] & 1 else 6 * nz[l] + 20 * rows[l]
-        cbytes = sum(2 * sweep_b(l) for l in range(1, L - 1)) + 4 * nc * ld + 8 * nc
+        cbytes = sum(2 * sweep_b(l) for l in range(1, L - 1)) + 4 * nc * ld + 8 * nc + (tail_b if pn else 0)
         out["amg_coarse"] = ("k_amg_pre / k_amg_post (CSR) and k_amg_sellp (pair-packed SELL-32), bfloat16 values, "
-                             "levels >= 1, and k_amg_dense",
-                             cbytes / (2 * (L - 2) + 1), "per V-cycle sum_l 2 (6 nnz_l + 20 n_l) (CSR) or "
-                                                         "2 (4 nnz_l + 16.5 n_l) (packed) + 4 nc ld + 8 nc, "
-                                                         "over 2(L-2)+1 launches")
+                             "levels >= 1, and k_resident_tail (the small levels) or k_amg_dense",
+                             cbytes / (2 * max(0, tail - 1) + 1), "per V-cycle sum_l 2 (6 nnz_l + 20 n_l) (CSR) or "
+                                                         "2 (4 nnz_l + 16.5 n_l) (packed) + 4 nc ld + 8 nc "
+                                                         "+ the shared launch's transfers, over 2 launches "
+                                                         "per level before it + 1")
     bcs = tuning.get("bicg_candidates")
     bc = bcs[tuning["bicg_chosen"] - 1] if bcs else {"lanes": 0}
     c16 = bool(bc.get("col16"))
@@ -395,6 +414,8 @@ def run_ours(args, rank, world):
     fam = {f: capi.oasis_profile_read(run_e.solver, f) for f in capi.PROF_FAMILIES}
     tun_e = capi.oasis_get_tuning(run_e.solver)
     amg_info = capi.oasis_get_amg_info(run_e.solver) if pc == capi.OASIS_PC_AMG else None
+    if amg_info:
+        amg_info["tail"] = amg_tail(amg_info)
     run_e.close()
     if net_e is not None:
         net_e.close()
@@ -511,8 +532,9 @@ def run_ours(args, rank, world):
     # and (all but the last) a correction, 5 per BiCGStab iteration; pressure: rhs
     # and guess 2, per sweep residual + CG start + (all but the last) correction,
     # 1 per CG iteration; update 1
-    # learned guess: input scales, inputs, two network layers, judge.  Multigrid:
-    # a V-cycle is 4 kernels per operator level + the dense coarsest solve; per
+    # learned guess: input scales, inputs, two network layers, judge.  A solve small
+    # enough to be resident is one launch.  Multigrid: a V-cycle is 4 kernels per
+    # operator level before the shared launch + that (or the dense coarsest solve); per
     # sweep residual, start, V-cycle, product, update (and all but the last a
     # correction); per further iteration of an inner solve (every sweep but the
     # last runs one) V-cycle, product, update.  Inner iterations
@@ -523,16 +545,22 @@ def run_ours(args, rank, world):
     # assembly, two residual sweeps and a correction, 5 per BiCGStab iteration,
     # the final update.
     if amg_info:
-        vk = 4 * (amg_info["levels"] - 1) + 1
+        vk = 4 * amg_info["tail"] + 1
         p_kernels = sw_p * (5 + vk) + max(0, it_p - (sw_p - 1)) * (2 + vk)
     else:
         p_kernels = 3 * sw_p + it_p
+    u_kernels = 2 * sw_u + 5 * it_u
+    small = pb.mesh.n_dofs <= RESIDENT_ROWS
+    if small:
+        u_kernels = 1
+    if small and (not amg_info or run.nnz <= RESIDENT_AMG_ENTRIES):
+        p_kernels = 3      # right-hand side, guess, solve
     ni = max(1, args.inner_iters)
     upd_kernels = 3 + 2 * it_m if args.velocity_update == "consistent" else 1
     upd_kernels += args.scalars * (5 + 5 * it_c)
     n_asm = 2 if args.convection == "abe" else 3
     n_asm += 1   # the tentative velocity u^I formed once per dof for the pressure right-hand side
-    launches = int(round(args.steps * (ni * (n_asm + 2 * sw_u + 5 * it_u + p_kernels) + (ni - 1)
+    launches = int(round(args.steps * (ni * (n_asm + u_kernels + p_kernels) + (ni - 1)
                                        + (5 if learned else 0) + upd_kernels)))
     run.close()
 
