@@ -77,11 +77,7 @@ def workload_config(name, pb, precision, gpu=True):
 # kernels as they stand (an entry is removed when its kernel changes)
 _S112 = "profiles/dram_traffic_products_stress112_rcm.md (stress112_rcm capture, scaled by algorithmic bytes)"
 MEASURED_TRAFFIC = {("stress128_rcm", "pcg_spmv@sell"): (215.0e6, _S112),
-                    ("stress128_rcm", "pcg_spmv@pairs"): (229.8e6, _S112),
-                    ("stress128_rcm", "amg_fine@pairs"): (163.3e6, _S112),
-                    ("stress128_rcm", "bicg_spmm@rows"): (332.4e6, _S112),
-                    ("stress128_rcm", "bicg_spmm@rows16"): (263.6e6, _S112)}
-
+                    ("stress128_rcm", "pcg_spmv@pairs"): (229.8e6, _S112)}
 
 # Sizes up to which the library runs a linear solve as one resident launch in the
 # captured step (kResidentRows, kResidentAmgEntries), and below which the V-cycle's
