@@ -620,6 +620,13 @@ void AmgWork::alloc(const AmgHierarchy& h, size_t vbytes) {
     }
     meet.alloc(resident_sync_bytes(0, 0));
     OASIS_CUDA(cudaMemset(meet.p, 0, meet.bytes()));
+    // the tail's levels run as separate kernels where the device does not take its launch
+    tail = 1;
+    while (tail < (int)L && h.lv[tail]->n > kTailRows) ++tail;
+    if (tail < (int)L) {
+        tail_plan = vbytes == 4 ? resident_plan_tail<float>(h.lv[tail]->n) : resident_plan_tail<double>(h.lv[tail]->n);
+        if (tail_plan.blocks == 0) tail = (int)L;
+    }
 }
 
 // ------------------------------------------------------------------ kernels
@@ -1118,8 +1125,7 @@ void amg_vcycle(const AmgHierarchy& h, AmgWork& wk, const V* r, V* u, KrylovStat
                 const ProfHook* prof) {
     const int L = (int)h.lv.size();
     // levels tail .. L - 1 and the dense one run in the tail's launch
-    int tail = 1;
-    while (tail < L && h.lv[tail]->n > kTailRows) ++tail;
+    const int tail = wk.tail;
     // the pair-packed copies serve the float32 cycle only
     auto sellp_ok = [](const AmgSellP& A) { return sizeof(V) == 4 && A.n > 0; };
     int ph = -1;

@@ -137,10 +137,21 @@ struct AmgHierarchy {
 // Build (once per mesh) from the assembled float64 K; no-op if present.
 void amg_build(Mesh& m, cudaStream_t s);
 
+// Launch shape of a resident solve.
+struct ResidentPlan {
+    int blocks = 0;                      // 0: separate kernels
+    int threads = 0, lanes = 0;          // lanes per row of the matrix products
+    int rows = 0, entries = 0;           // of one block at most
+    int smem = 0;                        // bytes
+    bool staged = false;                 // the matrix is copied to shared memory
+};
+
 // Per-solver work vectors of the V-cycle.
 struct AmgWork {
     std::vector<DBuf<double>> x, xo, res, rin;   // raw storage; viewed as V
     DBuf<unsigned char> meet;                    // where the tail's blocks meet
+    int tail = 1;                                // first level of the tail (the number of levels: no tail)
+    ResidentPlan tail_plan;
     void alloc(const AmgHierarchy& h, size_t vbytes);
 };
 

@@ -173,7 +173,7 @@ void spmv_dot_f64(const Mesh& m, const double* vals, const double* x, double* y,
 void noalloc_scratch(double** partial, uint32_t** ticket);
 int64_t noalloc_max_rows();
 
-int num_sms();
+int num_sms();                                 // of the current device
 // Blocks of `fn` (kBlock threads, no dynamic shared memory) resident on one SM of the
 // current device, from the occupancy calculator, cached per device and kernel: grids of
 // grid-stride kernels stay within one wave.

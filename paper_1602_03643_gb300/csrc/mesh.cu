@@ -14,12 +14,13 @@
 namespace oasis {
 
 int num_sms() {
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        OASIS_CUDA(cudaGetDevice(&dev));
-        OASIS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    }
+    static std::mutex mu;
+    static std::map<int, int> cache;
+    int dev = 0;
+    OASIS_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lock(mu);
+    int& sms = cache[dev];
+    if (!sms) OASIS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     return sms;
 }
 

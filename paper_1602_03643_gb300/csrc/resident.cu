@@ -839,6 +839,9 @@ enum ResCg {
     kCgAmg = 2       // multigrid
 };
 
+template <class P>
+constexpr int kJacobiForm = P::mixed ? kCgQuads : kCgJacobi;
+
 // Chronopoulos-Gear CG inside refinement sweeps: the method, stopping tests and
 // counters of the separate kernels (k_pcg_outer_sell, k_amg_cg_*, k_pcg_iter_sell;
 // step.cu).
@@ -1370,26 +1373,35 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_mass(StepData<
     gm.leave();
 }
 
-int smem_optin() {
-    int dev = 0, v = 0;
-    OASIS_CUDA(cudaGetDevice(&dev));
-    OASIS_CUDA(cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    return v;
-}
 // shared memory that the kernels hold statically (float64: the sums' slots)
 template <class P>
 constexpr int res_static(bool mass) {
     return (P::mixed ? 8 : mass ? 40 : 20) * 1024;
 }
 
+int device_attribute(cudaDeviceAttr what) {
+    int dev = 0, v = 0;
+    OASIS_CUDA(cudaGetDevice(&dev));
+    OASIS_CUDA(cudaDeviceGetAttribute(&v, what, dev));
+    return v;
+}
+// Whether the current device takes a cooperative launch of fn in this shape; sets the
+// kernel's shared-memory limit for the launches to come.
+template <class F>
+bool fits(F fn, const ResidentPlan& pl) {
+    if (!device_attribute(cudaDevAttrCooperativeLaunch)) return false;
+    cudaFuncAttributes fa{};
+    OASIS_CUDA(cudaFuncGetAttributes(&fa, fn));
+    const int most = device_attribute(cudaDevAttrMaxSharedMemoryPerBlockOptin) - (int)fa.sharedSizeBytes;
+    if (pl.smem > most) return false;
+    if (pl.smem > 0) OASIS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    int per_sm = 0;
+    OASIS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, pl.threads, (size_t)pl.smem));
+    return (int64_t)per_sm * num_sms() >= pl.blocks;
+}
+
 template <class... KArgs, class... Args>
 void launch(void (*fn)(KArgs...), const ResidentPlan& pl, cudaStream_t s, Args&&... args) {
-    if (pl.smem > 0) {
-        cudaFuncAttributes fa{};
-        OASIS_CUDA(cudaFuncGetAttributes(&fa, fn));
-        OASIS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        smem_optin() - (int)fa.sharedSizeBytes));
-    }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)pl.blocks);
     cfg.blockDim = dim3((unsigned)pl.threads);
@@ -1414,7 +1426,7 @@ ResidentPlan plan(const std::vector<int32_t>& row_ptr, int64_t n, int vectors, b
         p.entries = 0;
         for (int64_t lo = 0; lo < n; lo += p.rows)
             p.entries = std::max(p.entries, row_ptr[std::min<int64_t>(n, lo + p.rows)] - row_ptr[lo]);
-        const size_t vec = (size_t)vectors * res_vector_bytes<V>(p.rows), room = (size_t)(smem_optin() - res_static<P>(mass));
+        const size_t vec = (size_t)vectors * res_vector_bytes<V>(p.rows), room = (size_t)(device_attribute(cudaDevAttrMaxSharedMemoryPerBlockOptin) - res_static<P>(mass));
         const size_t mat = res_matrix_bytes<V>(p.rows, p.entries);
         if (vec > room) return false;
         p.staged = vec + mat <= room;
@@ -1443,20 +1455,6 @@ ResidentSync resident_sync(void* mem) {
     return {reinterpret_cast<uint32_t*>(p), reinterpret_cast<uint32_t*>(p + 256), p + 512, p + kSyncBytes};
 }
 
-template <class P>
-ResidentPlan resident_plan_bicg(const std::vector<int32_t>& row_ptr, int64_t n, int nr) {
-    return plan<P>(row_ptr, n, 6 * nr + 1);
-}
-template <class P>
-ResidentPlan resident_plan_mass(const std::vector<int32_t>& row_ptr, int64_t n, int d) {
-    return plan<P>(row_ptr, n, 5 * d + 2, true);
-}
-template <class P>
-ResidentPlan resident_plan_cg(const std::vector<int32_t>& row_ptr, int64_t n, bool amg) {
-    if (amg && row_ptr[n] > (P::mixed ? kResidentAmgEntries : kResidentAmgEntries64)) return {};
-    return plan<P>(row_ptr, n, 6);
-}
-
 // LAUNCH(lanes, entries in flight, staged) of a plan; a matrix that does not fit in
 // shared memory belongs to a plan with the fewest lanes
 #define OASIS_RES_SHAPE(LAUNCH)                                                              \
@@ -1466,6 +1464,51 @@ ResidentPlan resident_plan_cg(const std::vector<int32_t>& row_ptr, int64_t n, bo
     else if (pl.lanes >= 4) LAUNCH(4, 4, true);                                              \
     else if (pl.lanes >= 2) LAUNCH(kTwo, kM, true);                                          \
     else LAUNCH(kFew, kM, true)
+
+template <class P, int D, int NR>
+ResidentPlan resident_plan_bicg(const std::vector<int32_t>& row_ptr, int64_t n) {
+    const ResidentPlan pl = plan<P>(row_ptr, n, 6 * NR + 1);
+    bool ok = pl.blocks > 0;
+#define OASIS_RES_FITS(G, M, ST) ok = ok && fits(k_resident_bicg<P, D, NR, G, M, ST>, pl)
+    OASIS_RES_SHAPE(OASIS_RES_FITS);
+#undef OASIS_RES_FITS
+    return ok ? pl : ResidentPlan{};
+}
+template <class P, int D>
+ResidentPlan resident_plan_mass(const std::vector<int32_t>& row_ptr, int64_t n) {
+    const ResidentPlan pl = plan<P>(row_ptr, n, 5 * D + 2, true);
+    bool ok = pl.blocks > 0;
+#define OASIS_RES_FITS(G, M, ST) ok = ok && fits(k_resident_mass<P, D, G, M, ST>, pl)
+    OASIS_RES_SHAPE(OASIS_RES_FITS);
+#undef OASIS_RES_FITS
+    return ok ? pl : ResidentPlan{};
+}
+template <class P>
+ResidentPlan resident_plan_cg(const std::vector<int32_t>& row_ptr, int64_t n, bool amg) {
+    if (amg && row_ptr[n] > (P::mixed ? kResidentAmgEntries : kResidentAmgEntries64)) return {};
+    const ResidentPlan pl = plan<P>(row_ptr, n, 6);
+    bool ok = pl.blocks > 0;
+    if (amg) {
+#define OASIS_RES_FITS(G, M, ST) ok = ok && fits(k_resident_cg<P, G, M, kCgAmg, ST>, pl)
+        OASIS_RES_SHAPE(OASIS_RES_FITS);
+#undef OASIS_RES_FITS
+    } else {
+#define OASIS_RES_FITS(G, M, ST) ok = ok && fits(k_resident_cg<P, G, M, kJacobiForm<P>, ST>, pl)
+        OASIS_RES_SHAPE(OASIS_RES_FITS);
+#undef OASIS_RES_FITS
+    }
+    return ok ? pl : ResidentPlan{};
+}
+template <class V>
+ResidentPlan resident_plan_tail(int64_t n) {
+    ResidentPlan pl;
+    pl.threads = 512;
+    // at least 16 rows of the tail's finest level per block
+    pl.blocks = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(num_sms(), kResBlocks), (n + 15) / 16));
+    return !device_attribute(cudaDevAttrMpsEnabled) && fits(k_resident_tail<V>, pl) ? pl : ResidentPlan{};
+}
+template ResidentPlan resident_plan_tail<float>(int64_t);
+template ResidentPlan resident_plan_tail<double>(int64_t);
 
 template <class P, int D, int NR>
 void resident_bicg(const StepData<P>& q, int k0, const Ctl& c, const ResidentPlan& pl, const ResidentSync& sy,
@@ -1484,8 +1527,7 @@ void resident_cg(const StepData<P>& q, const Ctl& c, const ResidentAmg<typename 
         OASIS_RES_SHAPE(OASIS_RES_LAUNCH);
 #undef OASIS_RES_LAUNCH
     } else {
-        constexpr int kJacobi = P::mixed ? kCgQuads : kCgJacobi;
-#define OASIS_RES_LAUNCH(G, M, ST) launch(k_resident_cg<P, G, M, kJacobi, ST>, pl, s, q, c, m, pl, sy)
+#define OASIS_RES_LAUNCH(G, M, ST) launch(k_resident_cg<P, G, M, kJacobiForm<P>, ST>, pl, s, q, c, m, pl, sy)
         OASIS_RES_SHAPE(OASIS_RES_LAUNCH);
 #undef OASIS_RES_LAUNCH
     }
@@ -1555,10 +1597,7 @@ ResidentAmg<V> resident_amg(const AmgHierarchy& h, AmgWork& w, int first, int bl
 
 template <class V>
 void resident_tail(const AmgHierarchy& h, AmgWork& w, int first, KrylovState* st, cudaStream_t s) {
-    ResidentPlan pl;
-    pl.threads = 512;
-    // at least 16 rows of the tail's finest level per block
-    pl.blocks = (int)std::max<int64_t>(1, std::min<int64_t>(num_sms(), (h.lv[first]->n + 15) / 16));
+    const ResidentPlan& pl = w.tail_plan;
     launch(k_resident_tail<V>, pl, s, resident_amg<V>(h, w, first, pl.blocks, pl.threads), st, resident_sync(w.meet.p));
 }
 template void resident_tail<float>(const AmgHierarchy&, AmgWork&, int, KrylovState*, cudaStream_t);
@@ -1583,8 +1622,13 @@ template ResidentAmg<double> resident_amg<double>(const AmgHierarchy&, AmgWork&,
                                       const ResidentSync&, cudaStream_t);                                        \
     template void resident_cg<P>(const StepData<P>&, const Ctl&, const ResidentAmg<typename P::V>&,              \
                                  const ResidentPlan&, const ResidentSync&, cudaStream_t);                        \
-    template ResidentPlan resident_plan_bicg<P>(const std::vector<int32_t>&, int64_t, int);                      \
-    template ResidentPlan resident_plan_mass<P>(const std::vector<int32_t>&, int64_t, int);                      \
+    template ResidentPlan resident_plan_bicg<P, 3, 3>(const std::vector<int32_t>&, int64_t);                     \
+    template ResidentPlan resident_plan_bicg<P, 3, 1>(const std::vector<int32_t>&, int64_t);                     \
+    template ResidentPlan resident_plan_bicg<P, 2, 2>(const std::vector<int32_t>&, int64_t);                     \
+    template ResidentPlan resident_plan_bicg<P, 2, 1>(const std::vector<int32_t>&, int64_t);                     \
+    template ResidentPlan resident_plan_bicg<P, 1, 1>(const std::vector<int32_t>&, int64_t);                     \
+    template ResidentPlan resident_plan_mass<P, 3>(const std::vector<int32_t>&, int64_t);                        \
+    template ResidentPlan resident_plan_mass<P, 2>(const std::vector<int32_t>&, int64_t);                        \
     template ResidentPlan resident_plan_cg<P>(const std::vector<int32_t>&, int64_t, bool);
 OASIS_RES(Mixed)
 OASIS_RES(Fp64)

@@ -17,14 +17,6 @@ constexpr int kResBlocks = 1024;         // blocks of one launch at most
 // changed: 73^3 mixed 2890 / 3140, 621^2 mixed 2070 / 2320.
 constexpr int64_t kResidentRows = 650000;
 
-// Launch shape of a resident solve.
-struct ResidentPlan {
-    int blocks = 0;                      // 0: separate kernels
-    int threads = 0, lanes = 0;          // lanes per row of the matrix products
-    int rows = 0, entries = 0;           // of one block at most
-    int smem = 0;                        // bytes
-    bool staged = false;                 // the matrix is copied to shared memory
-};
 // Device memory in which the blocks of a launch meet (zero between launches).
 struct ResidentSync {
     uint32_t *count, *ticket;            // arrivals; blocks that have left
@@ -34,14 +26,20 @@ struct ResidentSync {
 size_t resident_sync_bytes(int64_t n, size_t value_bytes);
 ResidentSync resident_sync(void* mem);
 
-// Plans for the velocity solve of nr components, the mass solve of d and the pressure
-// solve on a pattern (host row pointers); blocks = 0 where a block's share does not fit.
-template <class P>
-ResidentPlan resident_plan_bicg(const std::vector<int32_t>& row_ptr, int64_t n, int nr);
-template <class P>
-ResidentPlan resident_plan_mass(const std::vector<int32_t>& row_ptr, int64_t n, int d);
+// Plans for the solve of NR of D components, the mass solve of D and the pressure solve
+// on a pattern (host row pointers), for the current device; blocks = 0 where a block's
+// share does not fit, or where the device does not take the launch (no cooperative
+// launches, or fewer blocks resident than the plan needs).
+template <class P, int D, int NR>
+ResidentPlan resident_plan_bicg(const std::vector<int32_t>& row_ptr, int64_t n);
+template <class P, int D>
+ResidentPlan resident_plan_mass(const std::vector<int32_t>& row_ptr, int64_t n);
 template <class P>
 ResidentPlan resident_plan_cg(const std::vector<int32_t>& row_ptr, int64_t n, bool amg);
+// Likewise for the tail of a V-cycle whose finest level has n rows.  The tail runs inside
+// conditional graph bodies, where cooperative launches are allowed without MPS only.
+template <class V>
+ResidentPlan resident_plan_tail(int64_t n);
 
 // One operator level of the multigrid cycle as a resident solve reads it.
 template <class V>

@@ -2476,7 +2476,8 @@ struct StepImplT final : StepImpl {
     double tune_us[OASIS_MAX_VARIANTS] = {0};
     int it_grid[OASIS_MAX_VARIANTS] = {0}, it_block[OASIS_MAX_VARIANTS] = {0};
     size_t it_smem[OASIS_MAX_VARIANTS] = {0};
-    ResidentPlan res_u{}, res_u1{}, res_m{}, res_p{}; // resident solves: D velocity components, one, mass, pressure
+    // resident solves: D velocity components, one, a scalar, mass, pressure
+    ResidentPlan res_u{}, res_u1{}, res_s{}, res_m{}, res_p{};
     ResidentSync res_sync{};
     ResidentAmg<V> res_amg{};
 
@@ -2659,11 +2660,16 @@ struct StepImplT final : StepImpl {
         ge_red = red_grid(m.n);
         ge_nd = elem_grid(m.n * D);
         ge_c = elem_grid(m.nc);
-        res_u = resident_plan_bicg<P>(m.h_row_ptr, m.n, D);
-        res_u1 = resident_plan_bicg<P>(m.h_row_ptr, m.n, 1);
-        res_m = resident_plan_mass<P>(m.h_row_ptr, m.n, D);
-        res_p = resident_plan_cg<P>(m.h_row_ptr, m.n, Sv.prm.pressure_pc == OASIS_PC_AMG);
-        if (res_u.blocks + res_u1.blocks + res_m.blocks + res_p.blocks > 0) {
+        // none where the caller forces a product shape
+        if (Sv.prm.bicg_variant == 0) {
+            if (Sv.prm.batch_rhs) res_u = resident_plan_bicg<P, D, D>(m.h_row_ptr, m.n);
+            else res_u1 = resident_plan_bicg<P, D, 1>(m.h_row_ptr, m.n);
+            res_s = resident_plan_bicg<P, 1, 1>(m.h_row_ptr, m.n);
+            if (Sv.prm.velocity_update == OASIS_UPDATE_CONSISTENT) res_m = resident_plan_mass<P, D>(m.h_row_ptr, m.n);
+        }
+        if (Sv.prm.spmv_variant == 0)
+            res_p = resident_plan_cg<P>(m.h_row_ptr, m.n, Sv.prm.pressure_pc == OASIS_PC_AMG);
+        if (res_u.blocks + res_u1.blocks + res_s.blocks + res_m.blocks + res_p.blocks > 0) {
             Sv.resident.alloc(resident_sync_bytes(m.n, sizeof(V)), nullptr);
             OASIS_CUDA(cudaStreamSynchronize(nullptr));
             res_sync = resident_sync(Sv.resident.p);
@@ -2677,10 +2683,10 @@ struct StepImplT final : StepImpl {
         }
     }
 
-    // Whether a solve with this plan runs resident: not where the caller forces a
-    // product shape or times kernel families (eager profiling).
-    bool resident(const ResidentPlan& pl, int32_t forced) const {
-        return pl.blocks > 0 && forced == 0 && !(Sv.prof_on && !Sv.prm.use_graph);
+    // Whether a solve with this plan runs resident: not where the caller times kernel
+    // families (eager profiling).
+    bool resident(const ResidentPlan& pl) const {
+        return pl.blocks > 0 && !(Sv.prof_on && !Sv.prm.use_graph);
     }
 
     void assemble(cudaStream_t s) override {
@@ -2726,8 +2732,8 @@ struct StepImplT final : StepImpl {
     // BiCGStab with refinement sweeps on the system of q (state index `which`).
     template <int DD, int NR>
     void bicg_run(const StepData<P>& q, cudaStream_t s, int which, int k0, bool graph) {
-        const ResidentPlan& pl = NR == 1 ? res_u1 : res_u;
-        if (resident(pl, Sv.prm.bicg_variant)) {
+        const ResidentPlan& pl = DD == 1 ? res_s : NR == 1 ? res_u1 : res_u;
+        if (resident(pl)) {
             resident_bicg<P, DD, NR>(q, k0, ctl_u(Loop{}), pl, res_sync, s);
             return;
         }
@@ -2856,7 +2862,7 @@ struct StepImplT final : StepImpl {
         Sv.prof_end(s, pg);
         k_phi_guess<P><<<ge_n, kBlock, 0, s>>>(a, mode);
         OASIS_CUDA(cudaGetLastError());
-        if (resident(res_p, Sv.prm.spmv_variant)) {
+        if (resident(res_p)) {
             resident_cg<P>(a, ctl_p(Loop{}), res_amg, res_p, res_sync, s);
             return;
         }
@@ -2948,7 +2954,7 @@ struct StepImplT final : StepImpl {
 
     void update(cudaStream_t s, bool graph) override {
         if (Sv.prm.velocity_update == OASIS_UPDATE_CONSISTENT) {
-            if (resident(res_m, Sv.prm.bicg_variant)) resident_mass<P, D>(a, Sv.prm.dt, ctl_m(Loop{}), res_m, res_sync, s);
+            if (resident(res_m)) resident_mass<P, D>(a, Sv.prm.dt, ctl_m(Loop{}), res_m, res_sync, s);
             else Sv.run_single(
                 s, graph, 2,
                 [&](cudaStream_t ss, const Loop& lp) {
