@@ -72,41 +72,117 @@ __device__ __forceinline__ A wider(ff a) { return a; }
 template <class T>
 using LiteA = typename LiteAcc<T>::type;
 
-// The Krylov scalars, computed by one thread between two meetings: float64, or in
-// the mixed path float-float, as the sums that they come from (a float64 operation
-// occupies the pipe for 64 cycles: the three quotients of a CG iteration took 1.4 us
-// in float64, measured).
-__device__ __forceinline__ double x_mul(double a, double b) { return a * b; }
-__device__ __forceinline__ double x_sub(double a, double b) { return a - b; }
-__device__ __forceinline__ double x_add(double a, double b) { return a + b; }
-__device__ __forceinline__ double x_div(double a, double b) { return a / b; }
+// The Krylov scalars.  Float64 path: float64.  Mixed path: what one iteration hands to
+// the next is exact (a grid-wide sum, float-float as it comes) or derived in float64 by
+// the block's last warp while the others go on; the coefficients that the vectors wait
+// for are float32 and come from quotients in float-float (a float64 operation occupies
+// the pipe for 64 cycles: a CG iteration with all of its scalars in float64 took 6.0 us
+// where it takes 5.3).  The sums may be as small as float32 holds: they are brought to
+// the order of one by a power of two first, and 1 / rho, which may be beyond float32, is
+// formed of the scaled rho only.
 __device__ __forceinline__ double x_hi(double a) { return a; }
+__device__ __forceinline__ float x_hi(ff a) { return a.hi; }
+__device__ __forceinline__ double x_mul(double a, double b) { return a * b; }
 __device__ __forceinline__ ff x_mul(ff a, ff b) {
     ff p = two_prod(a.hi, b.hi);
     p.lo = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, p.lo));
     return fast_two_sum(p.hi, p.lo);
 }
-__device__ __forceinline__ ff x_sub(ff a, ff b) { return ff_sub(a, b); }
-__device__ __forceinline__ ff x_add(ff a, ff b) { return ff_add(a, b); }
-// quotient to ~float-float accuracy: one correction by the exact remainder of the
-// float quotient (Dekker 1971)
+__device__ __forceinline__ double x_div(double a, double b) { return a / b; }
+// to ~float-float accuracy: one correction by the exact remainder of the float
+// quotient (Dekker 1971)
 __device__ __forceinline__ ff x_div(ff a, ff b) {
     const float q = a.hi / b.hi;
     const ff p = two_prod(q, b.hi);
     const float rem = ((a.hi - p.hi) - p.lo) + __fmaf_rn(-q, b.lo, a.lo);
     return fast_two_sum(q, rem / b.hi);
 }
-__device__ __forceinline__ float x_hi(ff a) { return a.hi; }
+// a power of two that brings a to the order of one (zero, infinity and NaN stay)
+__device__ __forceinline__ double unit_of(double) { return 1.0; }
+__device__ __forceinline__ float unit_of(ff a) {
+    return __uint_as_float((254u << 23) - min(__float_as_uint(a.hi) & 0x7f800000u, 253u << 23));
+}
+__device__ __forceinline__ double x_scaled(double a, double) { return a; }
+__device__ __forceinline__ ff x_scaled(ff a, float s) { return {a.hi * s, a.lo * s}; }
+// a / b as a value
 template <class X>
-__device__ __forceinline__ X x_of(double d);
+__device__ __forceinline__ auto quotient(X a, X b) {
+    const auto s = unit_of(b);
+    return x_hi(x_div(x_scaled(a, s), x_scaled(b, s)));
+}
+// the float64 limit of a sum's stopping test in the sum's leading type: not above it
+__device__ __forceinline__ double limit_of(double, double d) { return d; }
+__device__ __forceinline__ float limit_of(float, double d) { return __double2float_rd(d); }
+
+// What a CG iteration hands to the next: rho = <r, u> and 1 / alpha.
+template <class X>
+struct CgCarry;
 template <>
-__device__ __forceinline__ double x_of<double>(double d) { return d; }
+struct CgCarry<double> {
+    double rho, alpha, irho, ialpha;
+    // sweep's first product: alpha = rho / <w, u>
+    __device__ __forceinline__ double start(double g, double wu) {
+        rho = g;
+        return alpha = g / wu;
+    }
+    // beta = g / rho, alpha = g / (<w, u> - beta g / alpha_old); false: a breakdown
+    __device__ __forceinline__ bool next(double g, double wu, double& al, double& be) {
+        be = rho == 0.0 ? 0.0 : g * irho;
+        const double den = alpha == 0.0 ? 0.0 : wu - be * g * ialpha;
+        const bool ok = den > 0.0 && isfinite(den) && isfinite(g) && rho != 0.0;
+        al = alpha = ok ? g / den : 0.0;
+        rho = g;
+        return ok;
+    }
+    // between two iterations, off the critical path, by one warp: its lanes take a
+    // quotient each; g, wu: the sums that start or next had
+    __device__ __forceinline__ void carry(int lane, bool, double, double) {
+        const double q = 1.0 / (lane == 0 ? rho : alpha);
+        if (lane == 0 && rho != 0.0) irho = q;
+        if (lane == 1 && alpha != 0.0) ialpha = q;
+    }
+};
 template <>
-__device__ __forceinline__ ff x_of<ff>(double d) { return ff_from_double(d); }
-__device__ __forceinline__ bool x_zero(double a) { return a == 0.0; }
-__device__ __forceinline__ bool x_zero(ff a) { return a.hi == 0.f; }
-__device__ __forceinline__ bool x_finite(double a) { return isfinite(a); }
-__device__ __forceinline__ bool x_finite(ff a) { return isfinite(a.hi); }
+struct CgCarry<ff> {
+    ff rho, irho, ialpha;                // irho: of rho times unit; ialpha: of ia
+    float unit;
+    double ia;                           // 1 / alpha
+    __device__ __forceinline__ float start(ff g, ff wu) { return quotient(g, wu); }
+    __device__ __forceinline__ bool next(ff g, ff wu, float& al, float& be) {
+        const ff gs = x_scaled(g, unit), b = x_mul(gs, irho);
+        const ff den = ff_sub(x_scaled(wu, unit), x_mul(x_mul(b, gs), ialpha));
+        const bool ok = den.hi > 0.f && isfinite(den.hi) && isfinite(g.hi) && rho.hi != 0.f;
+        al = ok ? x_div(gs, den).hi : 0.f;
+        be = rho.hi != 0.f ? b.hi : 0.f;
+        return ok;
+    }
+    // 1 / alpha = <w, u> / g - (g / rho) / alpha_old
+    __device__ __forceinline__ void carry(int lane, bool first, ff g, ff wu) {
+        const float s = unit_of(g);
+        const ff num = lane == 0 ? wu : lane == 1 ? g : ff{1.f, 0.f};
+        const ff den = lane == 0 ? g : lane == 1 ? rho : x_scaled(g, s);
+        const double q = first && lane == 1 ? 0.0 : acc_double(num) / acc_double(den);
+        const double q1 = __shfl_sync(0xffffffffu, q, 1);
+        const double next_ia = first ? q : q - q1 * ia;
+        const ff f = ff_from_double(lane == 0 ? next_ia : q);
+        if (lane == 0) {
+            ia = next_ia;
+            ialpha = f;
+            rho = g;
+            unit = s;
+        }
+        if (lane == 2) irho = f;
+    }
+};
+// alpha / omega of a BiCGStab iteration, off the critical path: alpha = rho / <rhat, v>,
+// omega = <t, s> / <t, t>
+__device__ __forceinline__ double alpha_over_omega(double rho, double rv, double ts, double tt) {
+    return (rho / rv) / (ts / tt);
+}
+__device__ __forceinline__ ff alpha_over_omega(ff rho, ff rv, ff ts, ff tt) {
+    // float32's range: the products stay within float64's
+    return ff_from_double((acc_double(rho) * acc_double(tt)) / (acc_double(rv) * acc_double(ts)));
+}
 
 // ------------------------------------------------------------------ meetings
 __device__ __forceinline__ void add_release(uint32_t* p) {
@@ -424,18 +500,18 @@ struct BicgScalars {
     using X = LiteA<V>;
     X tot[kResValues];
     double bb[NR], rr[NR];
-    X rho[NR], alpha[NR], rr_in[NR];
-    V al[NR], om[NR], be[NR], stop[NR];  // stop: the inner solve ends at or below it
+    X rho[NR], rv[NR], ao[NR], rr_in[NR];   // <rhat, r>, <rhat, v>, alpha / omega, <r, r>
+    V al[NR], om[NR], be[NR], stop[NR];     // stop: the inner solve ends at or below it
     int it_total[NR], col_done[NR], in_done[NR], act[NR], status;
 };
 
 // Right-preconditioned BiCGStab with Jacobi inside refinement sweeps: the method,
 // the stopping tests and the counters of the separate kernels (k_bicg_*, step.cu).
-// Per iteration the blocks meet three times (mixed) or four (float64): after p and
-// ph; for <rhat, v>; [float64: after sh;] and for one sum that holds everything that
-// follows t: with r = s - omega t, <rhat, r> = <rhat, s> - omega <rhat, t> and
-// <r, r> = <s, s> - 2 omega <t, s> + omega^2 <t, t>, so that the update needs no sum
-// of its own.  The mixed path spares the meeting after sh as well: each neighbour's
+// Per iteration the blocks meet four times (mixed) or five (float64): after p and
+// ph; for <rhat, v>; [float64: after sh;] for <t, s> and <t, t>; and for <rhat, r> and
+// <r, r> of the new residual, summed from r itself (as differences of sums that come
+// with t, without a meeting of their own, they would lose the digits by which r is
+// smaller than s).  The mixed path spares the meeting after sh: each neighbour's
 // sh_j = d_j r_j - alpha d_j v_j is formed again from what is gathered; in float64
 // the extra arithmetic would cost more than the meeting.  Published, in pub: ph,
 // then (mixed) D^-1 r and D^-1 v, or (float64) sh.
@@ -472,11 +548,11 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_bicg(StepData<
     if (tid < NR) {
         sc.bb[tid] = st->bb[k0 + tid];
         sc.rr[tid] = st->rr[k0 + tid];
-        sc.rr_in[tid] = x_of<X>(0.0);
+        acc_zero(sc.rr_in[tid]);
         sc.col_done[tid] = st->col_done[k0 + tid];
         sc.in_done[tid] = 1;
         sc.it_total[tid] = st->it_total[k0 + tid];
-        sc.alpha[tid] = sc.rho[tid] = x_of<X>(0.0);
+        acc_zero(sc.rho[tid]);
         sc.al[tid] = sc.om[tid] = sc.be[tid] = V(0);
     }
     if (tid == 0) sc.status = st->status;
@@ -495,6 +571,7 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_bicg(StepData<
 #pragma unroll
         for (int c = 0; c < NR; ++c) acc[c] += av * g.v[c];
     };
+    const int spare = (int)blockDim.x - 32;
     // position of local element e = row * NR + c in an [n][D] array
     auto pos = [&](int e) { return (size_t)(ch.lo + e / NR) * D + k0 + e % NR; };
     bool ok = true;
@@ -544,7 +621,7 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_bicg(StepData<
             } else {
                 sc.in_done[tid] = 0;
                 sc.rho[tid] = sc.rr_in[tid] = sc.tot[tid];
-                sc.stop[tid] = (V)fmax(ctl.inner2 * rr, ctl.abs2 * sc.bb[tid]);
+                sc.stop[tid] = limit_of(V(0), fmax(ctl.inner2 * rr, ctl.abs2 * sc.bb[tid]));
             }
         }
         ++sweeps;
@@ -581,17 +658,17 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_bicg(StepData<
                 int act = !sc.col_done[tid] && !sc.in_done[tid];
                 if (act) {
                     const X rv = sc.tot[tid];
-                    if (x_zero(rv) || !x_finite(rv)) {
+                    if (x_hi(rv) == V(0) || !isfinite(x_hi(rv))) {
                         sc.in_done[tid] = 1;      // breakdown: restart from the float64-quality residual
                         sc.it_total[tid] += 1;
-                        sc.alpha[tid] = x_of<X>(0.0);
+                        sc.al[tid] = V(0);
                         act = 0;
                     } else {
-                        sc.alpha[tid] = x_div(sc.rho[tid], rv);
+                        sc.rv[tid] = rv;
+                        sc.al[tid] = quotient(sc.rho[tid], rv);
                     }
                 }
                 sc.act[tid] = act;
-                sc.al[tid] = x_hi(sc.alpha[tid]);
             }
             __syncthreads();
             if (!any_active()) break;
@@ -600,9 +677,9 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_bicg(StepData<
                     q1[ch.lo + e / NR].v[e % NR] = di[e / NR] * (r[e] - sc.al[e % NR] * v[e]);
                 if (!(ok = gm.barrier())) break;
             }
-            // t = A sh and the sums behind omega, <rhat, r> and <r, r>
+            // t = A sh, omega = <t, s> / <t, t>
             {
-                V part[5 * NR] = {};
+                V part[2 * NR] = {};
                 V al[NR];
 #pragma unroll
                 for (int c = 0; c < NR; ++c) al[c] = sc.al[c];
@@ -623,52 +700,71 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_bicg(StepData<
                         for (int c = 0; c < NR; ++c) {
                             if (c % G != lg) continue;
                             const int e = i * NR + c;
-                            const V tv = acc[c], hv = rh[e], sv = r[e] - al[c] * v[e];
+                            const V tv = acc[c], sv = r[e] - al[c] * v[e];
                             t[e] = tv;
                             part[c] += tv * sv;
                             part[NR + c] += tv * tv;
-                            part[2 * NR + c] += sv * sv;
-                            part[3 * NR + c] += hv * sv;
-                            part[4 * NR + c] += hv * tv;
                         }
                     });
-                if (!(ok = gm.template sum<5 * NR, NR, G, V, X>(part, sc.tot, used_groups<G>(rows)))) break;
+                if (!(ok = gm.template sum<2 * NR, NR, G, V, X>(part, sc.tot, groups))) break;
             }
             if (tid < NR && sc.act[tid]) {
-                const X ts = sc.tot[tid], tt = sc.tot[NR + tid], ss = sc.tot[2 * NR + tid];
-                const bool live = x_hi(tt) > V(0) && x_finite(tt);
-                const X om = live ? x_div(ts, tt) : x_of<X>(0.0);
-                const X rho = x_sub(sc.tot[3 * NR + tid], x_mul(om, sc.tot[4 * NR + tid]));
-                X rr = x_sub(ss, x_mul(om, x_sub(x_mul(ts, x_of<X>(2.0)), x_mul(om, tt))));
-                if (x_hi(rr) < V(0)) rr = x_of<X>(0.0);       // rounding; the sweep's own residual decides
+                const X ts = sc.tot[tid], tt = sc.tot[NR + tid];
+                sc.om[tid] = x_hi(tt) > V(0) && isfinite(x_hi(tt)) ? quotient(ts, tt) : V(0);
+            }
+            __syncthreads();
+            // off the critical path, by threads of the last warp
+            if (tid >= spare && tid < spare + NR) {
+                const int c = tid - spare;
+                if (sc.act[c]) sc.ao[c] = alpha_over_omega(sc.rho[c], sc.rv[c], sc.tot[c], sc.tot[NR + c]);
+            }
+            // delta += alpha ph + omega sh, r = s - omega t, <rhat, r>, <r, r>
+            {
+                V part[2 * NR] = {};
+                for (int i = tid / G; i < rows; i += (int)blockDim.x / G) {
+                    const int lg = tid % G;
+                    const V d = di[i];
+#pragma unroll
+                    for (int c = 0; c < NR; ++c) {
+                        if (c % G != lg || !sc.act[c]) continue;
+                        const int e = i * NR + c;
+                        const V al = sc.al[c], om = sc.om[c], sv = r[e] - al * v[e];
+                        dl[e] += al * (d * p[e]) + om * (d * sv);
+                        const V rv = sv - om * t[e];
+                        r[e] = rv;
+                        part[c] += rh[e] * rv;
+                        part[NR + c] += rv * rv;
+                    }
+                }
+                if (!(ok = gm.template sum<2 * NR, NR, G, V, X>(part, sc.tot, groups))) break;
+            }
+            if (tid < NR && sc.act[tid]) {
+                const X rho = sc.tot[tid], rr = sc.tot[NR + tid], old = sc.rho[tid];
                 sc.it_total[tid] += 1;
-                const X ro = x_mul(sc.rho[tid], om);
-                const X beta = x_zero(ro) ? x_of<X>(0.0) : x_div(x_mul(rho, sc.alpha[tid]), ro);
+                if (x_hi(old) != V(0) && sc.om[tid] != V(0)) {
+                    const auto s = unit_of(old);
+                    sc.be[tid] = x_hi(x_div(x_mul(x_scaled(rho, s), sc.ao[tid]), x_scaled(old, s)));
+                } else {
+                    sc.be[tid] = V(0);
+                }
                 sc.rho[tid] = rho;
                 sc.rr_in[tid] = rr;
-                sc.om[tid] = x_hi(om);
-                sc.be[tid] = x_hi(beta);
-                if (!x_finite(rr) || !x_finite(beta) || x_hi(rr) <= sc.stop[tid] || x_zero(om) || x_zero(rho) ||
+                if (!isfinite(x_hi(rr)) || x_hi(rr) <= sc.stop[tid] || sc.om[tid] == V(0) || x_hi(rho) == V(0) ||
                     sc.it_total[tid] >= ctl.max_it || it_in + 1 >= ctl.sweep_cap)
                     sc.in_done[tid] = 1;
             }
             ++it_in;
             __syncthreads();
-            // delta += alpha ph + omega sh, r = s - omega t, and the next p and ph
+            if (!any_active()) break;
+            // p = r + beta (p - omega v), ph = D^-1 p
             for (int e = tid; e < count; e += blockDim.x) {
                 const int row = e / NR, c = e % NR;
                 if (!sc.act[c]) continue;
-                const V d = di[row], vv = v[e], al = sc.al[c], om = sc.om[c], po = p[e];
-                const V sv = r[e] - al * vv;
-                dl[e] += al * (d * po) + om * (d * sv);
-                const V rv = sv - om * t[e];
-                r[e] = rv;
-                const V pv = rv + sc.be[c] * (po - om * vv);
+                const V d = di[row], rv = r[e], pv = rv + sc.be[c] * (p[e] - sc.om[c] * v[e]);
                 p[e] = pv;
                 ph[ch.lo + row].v[c] = d * pv;
                 if constexpr (P::mixed) q1[ch.lo + row].v[c] = d * rv;
             }
-            if (!any_active()) break;
         }
         if (!ok) break;
         // Delta += delta
@@ -702,11 +798,11 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_bicg(StepData<
 template <class V>
 struct CgScalars {
     using X = LiteA<V>;
-    X tot[kResValues];
+    X tot[kResValues], rr_in;
+    CgCarry<X> carry;
     double bb, rr;
-    X rr_in, rho, alpha, irho, ialpha;   // irho, ialpha: 1 / rho, 1 / alpha
     V al, be, stop;                      // stop: the inner solve ends at or below it
-    int it_total, col_done, in_done, last, status;   // last: the next update ends the inner solve
+    int it_total, col_done, in_done, status;
 };
 
 // One operator of the multigrid cycle on this block's rows, its entries read from
@@ -876,7 +972,7 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_cg(StepData<P>
         sc.it_total = st->it_total[0];
         sc.status = st->status;
         sc.rr = sc.bb = 0.0;
-        sc.rr_in = x_of<X>(0.0);
+        acc_zero(sc.rr_in);
     }
     int sweeps = st->sweeps, first = st->first, it_in = 0;
     double meanp = 0.0;
@@ -891,10 +987,9 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_cg(StepData<P>
     auto now = [] { return true; };
     auto add = [](V(&acc)[1], V kv, V x) { acc[0] += kv * x; };
     bool ok = true;
-    // u = M r (multigrid), then w = K u with <r, u>, <w, u>, <r, r> and (multigrid) the
-    // sums that give the next residual's norm; the meeting that makes r (Jacobi: u)
-    // visible comes first, unless the caller's sum was one
-    constexpr int kDots = MODE == kCgAmg ? 8 : 3;
+    // u = M r (multigrid), then w = K u with <r, u>, <w, u>, <r, r>; the meeting that
+    // makes r (Jacobi: u) visible comes first, unless the caller's sum was one
+    constexpr int kDots = 3;
     auto product = [&](bool met) {
         auto meet = [&] { return met || gm.barrier(); };
         if constexpr (MODE == kCgAmg) {
@@ -919,56 +1014,25 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_cg(StepData<P>
                     part[0] += rv * u;
                     part[1] += wv * u;
                     part[2] += rv * rv;
-                    if constexpr (MODE == kCgAmg) {
-                        const V sv = s[i];
-                        part[3] += rv * wv;
-                        part[4] += wv * wv;
-                        part[5] += rv * sv;
-                        part[6] += wv * sv;
-                        part[7] += sv * sv;
-                    }
                 }))
             return false;
         return gm.template sum<kDots, 1, G, V, X>(part, sc.tot, groups);
     };
-    // 1 / rho and 1 / alpha of the last iteration, off the critical path (by a thread
-    // of the last warp while the others start on the product)
-    const int spare = (int)blockDim.x - 32;
-    auto reciprocals = [&] {
-        if (tid == spare && !x_zero(sc.rho) && !x_zero(sc.alpha)) {
-            sc.irho = x_div(x_of<X>(1.0), sc.rho);
-            sc.ialpha = x_div(x_of<X>(1.0), sc.alpha);
-        }
-    };
-    // whether the update with alpha and beta meets the inner test, from
-    // r' = r - alpha (w + beta s): its norm needs no sum of its own
-    auto last = [&](X al, X be) {
-        const X two = x_of<X>(2.0);
-        const X rs = x_add(sc.tot[3], x_mul(be, sc.tot[5]));
-        const X ss = x_add(sc.tot[4], x_mul(be, x_add(x_mul(two, sc.tot[6]), x_mul(be, sc.tot[7]))));
-        const X rr = x_sub(sc.tot[2], x_mul(al, x_sub(x_mul(two, rs), x_mul(al, ss))));
-        sc.rr_in = rr;
-        return !x_finite(rr) || x_hi(rr) <= sc.stop || sc.it_total + 1 >= ctl.max_it || it_in + 1 >= ctl.sweep_cap;
+    // off the critical path (by the last warp while the others start on the product); the sums stay where they are until the blocks have met again
+    auto carry = [&] {
+        const int lane = tid - ((int)blockDim.x - 32);
+        if (lane >= 0) sc.carry.carry(lane, it_in == 0, sc.tot[0], sc.tot[1]);
     };
     // the coefficients of the next update, and the inner stopping test
     auto finish = [&] {
         ++it_in;
         if (tid == 0) {
-            const X g = sc.tot[0], rr = sc.tot[2];
+            const X rr = sc.tot[2];
             sc.it_total += 1;
-            // beta = g / g_old, alpha = g / (<w, u> - beta g / alpha_old)
-            const X b = x_zero(sc.rho) ? x_of<X>(0.0) : x_mul(g, sc.irho);
-            const X den = x_zero(sc.alpha) ? x_of<X>(0.0) : x_sub(sc.tot[1], x_mul(x_mul(b, g), sc.ialpha));
-            const bool brk = !(x_hi(den) > V(0)) || !x_finite(den) || !x_finite(g) || x_zero(sc.rho);
-            sc.alpha = brk ? x_of<X>(0.0) : x_div(g, den);
-            sc.rho = g;
+            const bool sound = sc.carry.next(sc.tot[0], sc.tot[1], sc.al, sc.be);
             sc.rr_in = rr;
-            sc.al = x_hi(sc.alpha);
-            sc.be = x_hi(b);
-            if (brk || !x_finite(rr) || x_hi(rr) <= sc.stop || sc.it_total >= ctl.max_it || it_in >= ctl.sweep_cap)
+            if (!sound || !isfinite(x_hi(rr)) || x_hi(rr) <= sc.stop || sc.it_total >= ctl.max_it || it_in >= ctl.sweep_cap)
                 sc.in_done = 1;
-            else if constexpr (MODE == kCgAmg)
-                sc.last = last(sc.alpha, b);
         }
         __syncthreads();
     };
@@ -1024,7 +1088,7 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_cg(StepData<P>
                     sc.col_done = 1;
                 } else {
                     sc.in_done = 0;
-                    sc.stop = (V)fmax(ctl.inner2 * rr, ctl.abs2 * sc.bb);
+                    sc.stop = limit_of(V(0), fmax(ctl.inner2 * rr, ctl.abs2 * sc.bb));
                 }
             }
         }
@@ -1038,17 +1102,13 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_cg(StepData<P>
         if (!(ok = product(true))) break;
         if (tid == 0) {
             const X g0 = sc.tot[0], d0 = sc.tot[1];
-            sc.alpha = x_of<X>(0.0);
-            if (!(x_hi(d0) > V(0)) || !x_finite(d0) || !x_finite(g0)) {
+            if (!(x_hi(d0) > V(0)) || !isfinite(x_hi(d0)) || !isfinite(x_hi(g0))) {
                 sc.in_done = 1;
                 sc.it_total += 1;
             } else {
-                sc.rho = g0;
-                sc.alpha = x_div(g0, d0);
+                sc.al = sc.carry.start(g0, d0);
             }
-            sc.al = x_hi(sc.alpha);
             sc.be = V(0);
-            if constexpr (MODE == kCgAmg) sc.last = !sc.in_done && last(sc.alpha, x_of<X>(0.0));
         }
         __syncthreads();
         if constexpr (MODE == kCgQuads) {
@@ -1057,7 +1117,7 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_cg(StepData<P>
         }
         while (!sc.in_done) {
             const V al = sc.al, be = sc.be;
-            reciprocals();
+            carry();
             if constexpr (MODE == kCgQuads) {
                 const Q* qo = (it_in & 1) ? a.pq0 : a.pq1;
                 Q* qn = (it_in & 1) ? a.pq1 : a.pq0;
@@ -1088,6 +1148,7 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_cg(StepData<P>
                 continue;
             }
             // p = u + beta p, s = w + beta s, delta += alpha p, r -= alpha s
+            V part[1] = {};
             for (int i = tid; i < rows; i += blockDim.x) {
                 const V u = MODE == kCgAmg ? a.au[ch.lo + i] : di[i] * r[i];
                 const V pv = be == V(0) ? u : u + be * p[i];
@@ -1097,22 +1158,32 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_cg(StepData<P>
                 dl[i] += al * pv;
                 const V rv = r[i] - al * sv;
                 r[i] = rv;
-                if constexpr (MODE == kCgAmg) a.ar[ch.lo + i] = rv;
-                else a.au[ch.lo + i] = di[i] * rv;
+                if constexpr (MODE == kCgAmg) {
+                    a.ar[ch.lo + i] = rv;
+                    part[0] += rv * rv;
+                } else {
+                    a.au[ch.lo + i] = di[i] * rv;
+                }
             }
             if constexpr (MODE == kCgAmg) {
-                // a residual that meets the inner test ends the solve before another cycle
-                if (sc.last) {
-                    __syncthreads();
-                    if (tid == 0) {
+                // a residual that meets the inner test ends the solve before another cycle;
+                // the sum is the meeting that makes r visible
+                if (!(ok = gm.template sum<1, 1, 1, V, X>(part, sc.tot, min(rows, (int)blockDim.x)))) break;
+                if (tid == 0) {
+                    const X rr = sc.tot[0];
+                    if (!isfinite(x_hi(rr)) || x_hi(rr) <= sc.stop || sc.it_total + 1 >= ctl.max_it || it_in + 1 >= ctl.sweep_cap) {
+                        sc.rr_in = rr;
                         sc.it_total += 1;
                         sc.in_done = 1;
                     }
+                }
+                __syncthreads();
+                if (sc.in_done) {
                     ++it_in;
                     break;
                 }
             }
-            if (!(ok = product(false))) break;
+            if (!(ok = product(MODE == kCgAmg))) break;
             finish();
         }
         if (!ok) break;
@@ -1276,8 +1347,8 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_mass(StepData<
             sc.rr[tid] = rr;
             sc.bb[tid] = bb;
             sc.be[tid] = V(0);
-            sc.stop[tid] = (V)(ctl.rtol2 * acc_double(bb));
-            if (!x_finite(rz) || !x_finite(rr) || !x_finite(bb)) sc.status = OASIS_ENAN;
+            sc.stop[tid] = limit_of(V(0), ctl.rtol2 * acc_double(bb));
+            if (!isfinite(x_hi(rz)) || !isfinite(x_hi(rr)) || !isfinite(x_hi(bb))) sc.status = OASIS_ENAN;
             sc.done[tid] = !(x_hi(rr) > sc.stop[tid]);
         }
         __syncthreads();
@@ -1308,12 +1379,12 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_mass(StepData<
         if (tid < D && !sc.done[tid]) {
             const X pq = sc.tot[tid];
             V al = V(0);
-            if (x_hi(pq) > V(0) && x_finite(pq)) {
-                al = x_hi(x_div(sc.rho[tid], pq));
+            if (x_hi(pq) > V(0) && isfinite(x_hi(pq))) {
+                al = quotient(sc.rho[tid], pq);
             } else {
                 // <p, q> = 0 with r != 0 cannot happen for SPD M: a breakdown
                 sc.done[tid] = 2;
-                sc.status = x_finite(pq) ? OASIS_EBREAKDOWN : OASIS_ENAN;
+                sc.status = isfinite(x_hi(pq)) ? OASIS_EBREAKDOWN : OASIS_ENAN;
             }
             sc.al[tid] = al;
         }
@@ -1339,13 +1410,13 @@ __global__ void __launch_bounds__(res_threads<P>(), 1) k_resident_mass(StepData<
         if (tid < D && !sc.done[tid]) {
             const X rz = sc.tot[tid], rr = sc.tot[D + tid];
             sc.rr[tid] = rr;
-            if (!x_finite(rz) || !x_finite(rr)) {
+            if (!isfinite(x_hi(rz)) || !isfinite(x_hi(rr))) {
                 sc.status = OASIS_ENAN;
                 sc.done[tid] = 1;
             } else if (!(x_hi(rr) > sc.stop[tid])) {
                 sc.done[tid] = 1;
             } else {
-                sc.be[tid] = x_hi(sc.rho[tid]) > V(0) ? x_hi(x_div(rz, sc.rho[tid])) : V(0);
+                sc.be[tid] = x_hi(sc.rho[tid]) > V(0) ? quotient(rz, sc.rho[tid]) : V(0);
                 sc.rho[tid] = rz;
             }
         }
