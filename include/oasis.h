@@ -475,7 +475,8 @@ int oasis_get_tuning(const oasis_solver* s, oasis_tuning* out);
 #define OASIS_PROF_PRESSURE_RHS 5  /* pressure right-hand side */
 #define OASIS_PROF_GUESS 6         /* learned guess: input scaling, network forward, judge */
 #define OASIS_PROF_AMG 7           /* multigrid V-cycles of the pressure CG */
-#define OASIS_PROF_MASS 8          /* consistent-mass update: the mass CG's start and iterations */
+#define OASIS_PROF_MASS 8          /* consistent-mass update: the mass CG's start and iterations
+                                      (one launch where the system is small enough) */
 /* Parts of OASIS_PROF_AMG (each V-cycle kernel is counted in one of them): */
 #define OASIS_PROF_AMG_FINE 9      /* smoothing sweeps of the finest level (the mesh's K) */
 #define OASIS_PROF_AMG_TRANSFER 10 /* restriction P^T and prolongation P, every level */
@@ -487,8 +488,15 @@ int oasis_get_tuning(const oasis_solver* s, oasis_tuning* out);
                                       tentative solve's r = r0 - A Delta and the pressure's
                                       r = b - K x) */
 
+/* Solves that run as one launch each (small systems): what would be the families 0, 1, 3,
+ * 7 and 9 to 13 of such a solve is inside that launch and not timed by itself. */
+#define OASIS_PROF_RESIDENT_BICG 14 /* a velocity solve (of all components, or of one with
+                                       batch_rhs = 0) or a scalar's solve */
+#define OASIS_PROF_RESIDENT_CG 15   /* the pressure solve */
+
 /* enable = 1: from now on, eager steps record CUDA events around the launches
- * of the kernel families above; the counters are reset by every call. */
+ * of the kernel families above; the counters are reset by every call.  The step
+ * launches the same kernels with and without. */
 int oasis_profile(oasis_solver* s, int32_t enable);
 
 /* Launch count and summed device time (ms) of one kernel family since the last

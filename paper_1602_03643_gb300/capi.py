@@ -356,7 +356,7 @@ def oasis_get_tentative_system(solver, dim, n, nnz, stream=None):
 
 PROF_FAMILIES = {"pcg_spmv": 0, "bicg_spmm": 1, "assemble": 2, "pcg_update": 3, "update": 4,
                  "pressure_rhs": 5, "guess": 6, "amg": 7, "mass": 8, "amg_fine": 9, "amg_transfer": 10,
-                 "amg_coarse": 11, "bicg_vec": 12, "outer": 13}
+                 "amg_coarse": 11, "bicg_vec": 12, "outer": 13, "resident_bicg": 14, "resident_cg": 15}
 
 
 def oasis_profile(solver, enable=True):

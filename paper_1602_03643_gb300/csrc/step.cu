@@ -2683,12 +2683,6 @@ struct StepImplT final : StepImpl {
         }
     }
 
-    // Whether a solve with this plan runs resident: not where the caller times kernel
-    // families (eager profiling).
-    bool resident(const ResidentPlan& pl) const {
-        return pl.blocks > 0 && !(Sv.prof_on && !Sv.prm.use_graph);
-    }
-
     void assemble(cudaStream_t s) override {
         const int pa = Sv.prof_begin(s, OASIS_PROF_ASSEMBLE);
         if (Sv.prm.convection == OASIS_CONV_ABE) {
@@ -2733,8 +2727,10 @@ struct StepImplT final : StepImpl {
     template <int DD, int NR>
     void bicg_run(const StepData<P>& q, cudaStream_t s, int which, int k0, bool graph) {
         const ResidentPlan& pl = DD == 1 ? res_s : NR == 1 ? res_u1 : res_u;
-        if (resident(pl)) {
+        if (pl.blocks > 0) {
+            const int pr = Sv.prof_begin(s, OASIS_PROF_RESIDENT_BICG);
             resident_bicg<P, DD, NR>(q, k0, ctl_u(Loop{}), pl, res_sync, s);
+            Sv.prof_end(s, pr);
             return;
         }
         const BicgGrids G = bicg_grids<DD, NR>();
@@ -2862,8 +2858,10 @@ struct StepImplT final : StepImpl {
         Sv.prof_end(s, pg);
         k_phi_guess<P><<<ge_n, kBlock, 0, s>>>(a, mode);
         OASIS_CUDA(cudaGetLastError());
-        if (resident(res_p)) {
+        if (res_p.blocks > 0) {
+            const int pq = Sv.prof_begin(s, OASIS_PROF_RESIDENT_CG);
             resident_cg<P>(a, ctl_p(Loop{}), res_amg, res_p, res_sync, s);
+            Sv.prof_end(s, pq);
             return;
         }
         if (Sv.prm.pressure_pc == OASIS_PC_AMG) {
@@ -2954,8 +2952,11 @@ struct StepImplT final : StepImpl {
 
     void update(cudaStream_t s, bool graph) override {
         if (Sv.prm.velocity_update == OASIS_UPDATE_CONSISTENT) {
-            if (resident(res_m)) resident_mass<P, D>(a, Sv.prm.dt, ctl_m(Loop{}), res_m, res_sync, s);
-            else Sv.run_single(
+            if (res_m.blocks > 0) {
+                const int pm = Sv.prof_begin(s, OASIS_PROF_MASS);
+                resident_mass<P, D>(a, Sv.prm.dt, ctl_m(Loop{}), res_m, res_sync, s);
+                Sv.prof_end(s, pm);
+            } else Sv.run_single(
                 s, graph, 2,
                 [&](cudaStream_t ss, const Loop& lp) {
                     const int pm = Sv.prof_begin(ss, OASIS_PROF_MASS);
