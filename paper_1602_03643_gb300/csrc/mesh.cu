@@ -560,6 +560,56 @@ __global__ void __launch_bounds__(kBlock) k_spmv(int64_t n, const int32_t* __res
     }
 }
 
+// A lane's share of a row's sum.  Eight entries added one after the other would round
+// more than 16 lanes with one entry each and a tree over them do.  Float32: the rounding
+// errors of products and sums are kept beside the sum (two_sum, the product's error by an
+// FMA) and added once at the end; where the sum is not finite it stands by itself.
+// Float64, whose pipe has no room for that: four sums taken in turn, then a tree (with the
+// dot one sum: the tiles of 256 rows that it replaces added a row's entries in sequence).
+template <class V, int NA>
+struct RowSum {
+    V s[NA];
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int k = 0; k < NA; ++k) s[k] = 0;
+    }
+    __device__ __forceinline__ void add(int k, V a, V x) { s[k] += a * x; }
+    template <int G>
+    __device__ __forceinline__ V total() {
+#pragma unroll
+        for (int h = NA / 2; h > 0; h /= 2)
+#pragma unroll
+            for (int k = 0; k < h; ++k) s[k] += s[k + h];
+        return group_sum<G>(s[0]);
+    }
+};
+template <int NA>
+struct RowSum<float, NA> {
+    float s, lo;
+    __device__ __forceinline__ void zero() { s = lo = 0.f; }
+    // s + x and its rounding error (Knuth, TAOCP vol. 2, 4.2.2)
+    __device__ __forceinline__ void add(float x) {
+        const float t = s + x, b = t - s;
+        lo += (s - (t - b)) + (x - b);
+        s = t;
+    }
+    __device__ __forceinline__ void add(int, float a, float x) {
+        const float p = a * x;
+        lo += __fmaf_rn(a, x, -p);
+        add(p);
+    }
+    template <int G>
+    __device__ __forceinline__ float total() {
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) {
+            const float other = __shfl_xor_sync(0xffffffffu, lo, o);
+            add(__shfl_xor_sync(0xffffffffu, s, o));
+            lo += other;
+        }
+        return isfinite(lo) ? s + lo : s;
+    }
+};
+
 // The library's own choice: G lanes per row and U rows in flight per lane group (row
 // pointers, then one entry of every row per round), the grid one resident wave; columns
 // as the pattern's 16-bit offsets from the row, modulo n, where it has them (C16: 6
@@ -569,8 +619,10 @@ __global__ void __launch_bounds__(kBlock) k_spmv(int64_t n, const int32_t* __res
 // Bound by the dependent loads row pointer -> column -> operand, so rows in flight
 // count.  1,030,200 rows, 15.2 M entries in reverse Cuthill-McKee order, one product
 // each with M in float64, K in float32 and K in float64 with the dot: 393 us with 16
-// lanes per row and one row at a time (DOT: 256-row tiles through shared memory), 160
-// with this form; the bytes alone take 72 at the copy rate.
+// lanes per row and one row at a time (DOT: 256-row tiles through shared memory), 170
+// with this form (160 with one plain sum per lane, whose errors were 3 to 7 % larger than
+// those of 16 lanes; 6.4e-8 against 3.9e-8 in float32); the bytes alone take 72 at the
+// copy rate.
 template <class V, int G, int U, bool C16, bool DOT>
 __global__ void __launch_bounds__(kBlock) k_spmv_rows(int64_t n, const int32_t* __restrict__ rp,
                                                       const int32_t* __restrict__ col,
@@ -579,6 +631,7 @@ __global__ void __launch_bounds__(kBlock) k_spmv_rows(int64_t n, const int32_t* 
                                                       double* __restrict__ partial, uint32_t* ticket,
                                                       double* __restrict__ xy) {
     constexpr int RPW = 32 / G;
+    constexpr int NA = sizeof(V) == 8 && !DOT ? 4 : 1;
     const int lane = threadIdx.x & 31, lg = lane & (G - 1), grp = lane / G;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -587,51 +640,55 @@ __global__ void __launch_bounds__(kBlock) k_spmv_rows(int64_t n, const int32_t* 
     for (int64_t base = w0 * RPW * U; base < n; base += nw * RPW * U) {
         uint32_t i[U];
         int32_t q[U], e[U];
-        V acc[U];
+        RowSum<V, NA> acc[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             i[u] = (uint32_t)(base + u * RPW + grp);
             const bool ok = i[u] < n32;
             q[u] = ok ? rp[i[u]] + lg : 0;
             e[u] = ok ? rp[i[u] + 1] : 0;
-            acc[u] = 0;
+            acc[u].zero();
         }
         bool more = false;
 #pragma unroll
         for (int u = 0; u < U; ++u) more |= q[u] < e[u];
         while (more) {
-            uint32_t j[U];
-            V av[U], g[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const bool has = q[u] < e[u];
-                uint32_t jc = 0;
-                if constexpr (C16) {
-                    // row + offset, wrapped once into [0, n)
-                    int32_t jj = (int32_t)i[u] + (int32_t)(has ? dcol[q[u]] : (int16_t)0);
-                    jj = jj < 0 ? jj + (int32_t)n32 : jj;
-                    jc = (uint32_t)jj >= n32 ? (uint32_t)jj - n32 : (uint32_t)jj;
-                } else {
-                    jc = has ? (uint32_t)col[q[u]] : 0u;
+            for (int turn = 0; turn < NA; ++turn) {
+                if (turn > 0 && !more) break;
+                uint32_t j[U];
+                V av[U], g[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const bool has = q[u] < e[u];
+                    uint32_t jc = 0;
+                    if constexpr (C16) {
+                        // row + offset, wrapped once into [0, n)
+                        int32_t jj = (int32_t)i[u] + (int32_t)(has ? dcol[q[u]] : (int16_t)0);
+                        jj = jj < 0 ? jj + (int32_t)n32 : jj;
+                        jc = (uint32_t)jj >= n32 ? (uint32_t)jj - n32 : (uint32_t)jj;
+                    } else {
+                        jc = has ? (uint32_t)col[q[u]] : 0u;
+                    }
+                    j[u] = has ? jc : 0u;
+                    av[u] = has ? val[q[u]] : V(0);
                 }
-                j[u] = has ? jc : 0u;
-                av[u] = has ? val[q[u]] : V(0);
-            }
 #pragma unroll
-            for (int u = 0; u < U; ++u) g[u] = x[j[u]];
-            more = false;
+                for (int u = 0; u < U; ++u) g[u] = x[j[u]];
+                more = false;
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                if (q[u] < e[u]) {
-                    acc[u] += av[u] * g[u];
-                    q[u] += G;
+                for (int u = 0; u < U; ++u) {
+                    if (q[u] < e[u]) {
+                        acc[u].add(turn, av[u], g[u]);
+                        q[u] += G;
+                    }
+                    more |= q[u] < e[u];
                 }
-                more |= q[u] < e[u];
             }
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const V sum = group_sum<G>(acc[u]);
+            const V sum = acc[u].template total<G>();
             if (i[u] < n32 && lg == 0) {
                 y[i[u]] = sum;
                 if constexpr (DOT) dot[0] += x[i[u]] * sum;

@@ -1,0 +1,61 @@
+"""Rounding errors of the stand-alone products with the library's own shape (lanes = 0).
+
+Measured against sums in extended precision, over a mesh with ~15 entries per row, beside
+16 lanes per row (one entry per lane and a tree of four additions, every product rounded).
+A lane of the library's shape takes eight entries: it must not round more than that.  Over
+68,921 rows the root mean square of the errors is known to better than a percent; 2 % are
+allowed for it.  Infinities and NaN in the operand come out as in the plain sum.
+"""
+import numpy as np
+import pytest
+
+from test_gpu_resident import _lib  # noqa: F401
+from workloads import meshes as WM
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("order", ["rcm", "random"])
+def test_own_shape_rounds_no_more_than_16_lanes(order):
+    import torch
+    from paper_1602_03643_gb300 import capi as c
+    m = WM.jitter_interior(WM.box_mesh_3d(40, 40, 40), 0.15, 1 / 40, 3)
+    perm = WM.rcm_permutation(m) if order == "rcm" else WM.random_permutation(m.n_dofs, 8)
+    h = c.oasis_mesh_create(m.dim, m.coords, m.cells, m.dof_of_vertex, m.n_dofs, perm)
+    try:
+        c.oasis_assemble_constant(h)
+        rp, col = c.oasis_mesh_get_pattern(h)
+        x = np.random.default_rng(2).normal(size=m.n_dofs)
+        for dt, spmv in ((np.float64, c.oasis_spmv_f64), (np.float32, c.oasis_spmv_f32)):
+            xi = np.empty(m.n_dofs, dt)
+            xi[perm] = x.astype(dt)
+            X = torch.from_numpy(xi).cuda()
+            wide = np.longdouble if dt is np.float64 else np.float64
+            for which in (c.OASIS_MAT_M, c.OASIS_MAT_K, c.OASIS_MAT_G0):
+                v = c.oasis_mesh_get_matrix(h, which).astype(dt).astype(wide)
+                want = np.add.reduceat(v * x.astype(dt).astype(wide)[col], rp[:-1])
+                rms = []
+                for lanes in (0, 16):
+                    Y = torch.empty_like(X)
+                    spmv(h, which, X, Y, lanes)
+                    torch.cuda.synchronize()
+                    rms.append(float(np.sqrt(np.mean((Y.cpu().numpy()[perm].astype(wide) - want) ** 2))))
+                assert rms[0] <= 1.02 * rms[1], (which, dt, rms)
+        # the columns of one row reach its neighbours: infinities and NaN as in the plain sum
+        for bad in (np.inf, -np.inf, np.nan):
+            xb = x.astype(np.float32)
+            xb[1234] = bad
+            xi = np.empty_like(xb)
+            xi[perm] = xb
+            X = torch.from_numpy(xi).cuda()
+            Y = [torch.empty_like(X) for _ in range(2)]
+            for y, lanes in zip(Y, (0, 16)):
+                c.oasis_spmv_f32(h, c.OASIS_MAT_M, X, y, lanes)
+            torch.cuda.synchronize()
+            a, b = (y.cpu().numpy() for y in Y)
+            hit = ~np.isfinite(b)
+            assert hit.any()
+            np.testing.assert_array_equal(a[hit], b[hit])
+            assert np.isfinite(a[~hit]).all()
+    finally:
+        c.oasis_mesh_destroy(h)
