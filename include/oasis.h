@@ -455,8 +455,14 @@ int oasis_get_amg_info(const oasis_solver* s, oasis_amg_info* out);
 
 /* u = M r with one V-cycle of the solver's hierarchy, in the solver's inner
  * precision (float64 for OASIS_FP64, float32 for OASIS_MIXED); r, u device
- * arrays of n_dofs values.  Synchronises `stream`.  Test hook. */
+ * arrays of n_dofs values.  Synchronises `stream`; OASIS_EWAIT if a bounded wait
+ * of its launches ran out (u is then incomplete).  Test hook. */
 int oasis_amg_apply(oasis_solver* s, const void* r, void* u, void* stream);
+
+/* Limit of the bounded waits in which the blocks of this solver's launches meet, in SM
+ * clock cycles from the next launch on (0: the usual ~2 s).  Waits for `stream`, on which
+ * the solver's earlier steps must have run.  Test hook. */
+int oasis_set_wait_limit(oasis_solver* s, int64_t cycles, void* stream);
 
 /* What the autotuner of oasis_solver_create chose for this solver. */
 int oasis_get_tuning(const oasis_solver* s, oasis_tuning* out);

@@ -132,6 +132,7 @@ SIGNATURES = {
     "oasis_get_scalar_fields": (C.c_int, [P, DPTR, I32, P]),
     "oasis_set_scalar_dirichlet": (C.c_int, [P, DPTR, I32, P]),
     "oasis_get_tentative_system": (C.c_int, [P, DPTR, DPTR, P]),
+    "oasis_set_wait_limit": (C.c_int, [P, I64, P]),
     "oasis_profile": (C.c_int, [P, I32]),
     "oasis_profile_read": (C.c_int, [P, I32, C.POINTER(I64), C.POINTER(C.c_double)]),
     "oasis_net_create": (C.c_int, [P, PP]),
@@ -434,6 +435,10 @@ def oasis_get_amg_info(solver):
 
 def oasis_amg_apply(solver, r, u, stream=None):
     check(lib().oasis_amg_apply(solver, _ptr(r), _ptr(u), _stream(stream)))
+
+
+def oasis_set_wait_limit(solver, cycles, stream=None):
+    check(lib().oasis_set_wait_limit(solver, int(cycles), _stream(stream)))
 
 
 def oasis_solver_destroy(solver):

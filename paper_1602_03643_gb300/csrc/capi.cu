@@ -10,6 +10,7 @@
 #include "solver.cuh"
 #include "kern.cuh"
 #include "amg.cuh"
+#include "resident.cuh"
 #include "net.cuh"
 
 namespace oasis {
@@ -713,6 +714,16 @@ int oasis_get_tentative_system(oasis_solver* solver, double* A_values, double* r
             OASIS_CUDA(cudaMemcpyAsync(r0, S->stage.p, n * D * sizeof(double), cudaMemcpyDeviceToHost, s));
         }
         OASIS_CUDA(cudaStreamSynchronize(s));
+    });
+}
+
+int oasis_set_wait_limit(oasis_solver* solver, int64_t cycles, void* stream) {
+    return guarded([&] {
+        Solver* S = reinterpret_cast<Solver*>(solver);
+        OASIS_CHECK(S, OASIS_EINVAL, "null solver");
+        OASIS_CHECK(cycles >= 0, OASIS_EINVAL, "a wait limit is not negative");
+        for (void* mem : {S->resident.p, (void*)S->amgw.meet.p})
+            if (mem) resident_set_wait(mem, cycles, as_stream(stream));
     });
 }
 

@@ -195,16 +195,18 @@ __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
 }
 
 // Every block's writes so far become visible to every block; false in all threads
-// of a block whose wait ran out.  goal: arrivals that the meeting waits for.
+// of a block whose wait ran out.  goal: arrivals that the meeting waits for.  The limit
+// of a wait, if not the usual one, stands behind the counter (resident_set_wait).
 __device__ __forceinline__ bool grid_barrier(uint32_t* count, uint32_t goal) {
     __syncthreads();
     bool ok = true;
     if (threadIdx.x == 0) {
         add_release(count);
         if ((int32_t)(ld_acquire(count) - goal) < 0) {
-            const long long t0 = clock64();
+            const long long t0 = clock64(), set = *reinterpret_cast<const volatile long long*>(count + 2),
+                            limit = set > 0 ? set : kBarrierLimitCycles;
             while ((int32_t)(ld_acquire(count) - goal) < 0)
-                if (clock64() - t0 > kBarrierLimitCycles) {
+                if (clock64() - t0 > limit) {
                     ok = false;
                     break;
                 }
@@ -1535,6 +1537,11 @@ ResidentSync resident_sync(void* mem) {
     else if (pl.lanes >= 4) LAUNCH(4, 4, true);                                              \
     else if (pl.lanes >= 2) LAUNCH(kTwo, kM, true);                                          \
     else LAUNCH(kFew, kM, true)
+
+void resident_set_wait(void* mem, int64_t cycles, cudaStream_t s) {
+    OASIS_CUDA(cudaMemcpyAsync(static_cast<unsigned char*>(mem) + 8, &cycles, sizeof(cycles), cudaMemcpyHostToDevice, s));
+    OASIS_CUDA(cudaStreamSynchronize(s));
+}
 
 template <class P, int D, int NR>
 ResidentPlan resident_plan_bicg(const std::vector<int32_t>& row_ptr, int64_t n) {

@@ -25,6 +25,8 @@ struct ResidentSync {
 };
 size_t resident_sync_bytes(int64_t n, size_t value_bytes);
 ResidentSync resident_sync(void* mem);
+// Limit of the waits of launches that meet there, in SM clock cycles (0: the usual one).
+void resident_set_wait(void* mem, int64_t cycles, cudaStream_t s);
 
 // Plans for the solve of NR of D components, the mass solve of D and the pressure solve
 // on a pattern (host row pointers), for the current device; blocks = 0 where a block's

@@ -3300,7 +3300,10 @@ struct StepImplT final : StepImpl {
         OASIS_CUDA(cudaMemsetAsync(scratch.p, 0, sizeof(KrylovState), s));
         amg_vcycle<V>(*Sv.m->amg, Sv.amgw, reinterpret_cast<const V*>(r), reinterpret_cast<V*>(u), scratch.p, s,
                       false);
+        KrylovState end;
+        OASIS_CUDA(cudaMemcpyAsync(&end, scratch.p, sizeof(end), cudaMemcpyDeviceToHost, s));
         OASIS_CUDA(cudaStreamSynchronize(s));
+        OASIS_CHECK(end.status == OASIS_OK, end.status, "a wait of the V-cycle's launch ran out");
     }
 
     void guess_target(cudaStream_t s, float* target) override {
