@@ -620,6 +620,8 @@ void AmgWork::alloc(const AmgHierarchy& h, size_t vbytes) {
     }
     meet.alloc(resident_sync_bytes(0, 0));
     OASIS_CUDA(cudaMemset(meet.p, 0, meet.bytes()));
+    // the solver's stream need not wait for the stream of these
+    OASIS_CUDA(cudaStreamSynchronize(nullptr));
     // the tail's levels run as separate kernels where the device does not take its launch
     tail = 1;
     while (tail < (int)L && h.lv[tail]->n > kTailRows) ++tail;

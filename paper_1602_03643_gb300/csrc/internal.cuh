@@ -72,9 +72,13 @@ struct DBuf {
         p = nullptr;
         n = 0;
     }
+    // The host array may go when this returns: it waits for the copy (the runtime need not
+    // stage pageable memory that the device reads itself, and copies later then).
     void upload(const T* host, size_t count, cudaStream_t s) {
         alloc(count);
-        if (count) OASIS_CUDA(cudaMemcpyAsync(p, host, count * sizeof(T), cudaMemcpyHostToDevice, s));
+        if (!count) return;
+        OASIS_CUDA(cudaMemcpyAsync(p, host, count * sizeof(T), cudaMemcpyHostToDevice, s));
+        OASIS_CUDA(cudaStreamSynchronize(s));
     }
     size_t bytes() const { return n * sizeof(T); }
 };
