@@ -628,7 +628,7 @@ __device__ __forceinline__ void bicg_dir_rows(const StepData<P>& a, int k0, int6
     p.store(a.p, row, k0, act);
 }
 template <class P, int D, int NR>
-__global__ void __launch_bounds__(kBlock) k_bicg_dir(StepData<P> a, int k0) {
+__global__ void __launch_bounds__(kBlock, 1) k_bicg_dir(StepData<P> a, int k0) {
     using V = typename P::V;
     constexpr int R = bicg_rows_per_thread<V, D, NR>();
     int act[NR];
@@ -854,13 +854,27 @@ static const BicgVariant<P, D>* bicg_variant_table() {
 #define OASIS_BICGV(G, U, B, C)                                                                              \
     {k_bicg_spmm_rows<P, D, D, 0, G, U, B, C>, k_bicg_spmm_rows<P, D, D, 1, G, U, B, C>,                    \
      k_bicg_outer_rows<P, D, D, G, 2>, G, U, B, C}
-    static const BicgVariant<P, D> t[kBicgVariants] = {
-        {k_bicg_spmm<P, D, D, 0, kTileN>, k_bicg_spmm<P, D, D, 1, kTileN>, nullptr, 0, kTileN, 1, 0},
-        OASIS_BICGV(4, 4, 1, false), OASIS_BICGV(4, 4, 5, false), OASIS_BICGV(2, 4, 1, false),
-        OASIS_BICGV(2, 4, 5, false), OASIS_BICGV(4, 4, 1, true), OASIS_BICGV(4, 4, 5, true),
-        OASIS_BICGV(2, 4, 1, true)};
+#define OASIS_BICG_TILE {k_bicg_spmm<P, D, D, 0, kTileN>, k_bicg_spmm<P, D, D, 1, kTileN>, nullptr, 0, kTileN, 1, 0}
+    if constexpr (P::mixed) {
+        static const BicgVariant<P, D> t[kBicgVariants] = {
+            OASIS_BICG_TILE, OASIS_BICGV(4, 4, 1, false), OASIS_BICGV(4, 4, 5, false), OASIS_BICGV(2, 4, 1, false),
+            OASIS_BICGV(2, 4, 5, false), OASIS_BICGV(4, 4, 1, true), OASIS_BICGV(4, 4, 5, true),
+            OASIS_BICGV(2, 4, 1, true)};
+        return t;
+    } else {
+        // No float64 shape caps its registers: for 5 blocks per SM they spilled 150-300
+        // bytes, and steps with such a shape raised "misaligned address" (79,507 rows, 2
+        // lanes; the same step runs with each shape below).  Two rows in flight need fewer
+        // registers by themselves.  us per pair of products, capped / not: 79,507 rows 67.3
+        // / 67.5, 132,651 rows 70.6 / 71.3; 4 lanes 75.4 / 71.1, 97.4 / 85.4.
+        static const BicgVariant<P, D> t[kBicgVariants] = {
+            OASIS_BICG_TILE, OASIS_BICGV(4, 4, 1, false), OASIS_BICGV(4, 2, 1, false), OASIS_BICGV(2, 4, 1, false),
+            OASIS_BICGV(2, 2, 1, false), OASIS_BICGV(4, 4, 1, true), OASIS_BICGV(4, 2, 1, true),
+            OASIS_BICGV(2, 4, 1, true)};
+        return t;
+    }
+#undef OASIS_BICG_TILE
 #undef OASIS_BICGV
-    return t;
 }
 
 // s = r - alpha v,  sh = D^{-1} s
@@ -1934,7 +1948,8 @@ static const AmgVariant<P>* amg_variant_table(int& count) {
         count = (int)(sizeof(t) / sizeof(t[0]));
         return t;
     } else {
-        static const AmgVariant<P> t[] = {OASIS_AMGV(4, 1), OASIS_AMGV(2, 8), OASIS_AMGV(4, 8), OASIS_AMGV(8, 4)};
+        // (for 8 blocks per SM the float64 registers spilled)
+        static const AmgVariant<P> t[] = {OASIS_AMGV(4, 1), OASIS_AMGV(2, 4), OASIS_AMGV(4, 4), OASIS_AMGV(8, 4)};
         count = (int)(sizeof(t) / sizeof(t[0]));
         return t;
     }
