@@ -79,16 +79,18 @@ _S112 = "profiles/dram_traffic_products_stress112_rcm.md (stress112_rcm capture,
 MEASURED_TRAFFIC = {("stress128_rcm", "pcg_spmv@sell"): (215.0e6, _S112),
                     ("stress128_rcm", "pcg_spmv@pairs"): (229.8e6, _S112)}
 
-# Sizes up to which the library runs a linear solve as one resident launch in the
-# captured step (kResidentRows, kResidentAmgEntries), and below which the V-cycle's
-# levels share one launch (kTailRows)
-RESIDENT_ROWS, RESIDENT_AMG_ENTRIES, TAIL_ROWS = 650_000, 1_900_000, 40_000
+def amg_tail(amg, fam):
+    """First level of the V-cycle's shared launch (the number of operator levels if none),
+    from the launches that a profiled step made: each level before it has two transfers."""
+    cycles, transfers = fam["amg"][0], fam["amg_transfer"][0]
+    return transfers // (2 * cycles) if cycles else amg["levels"] - 1
 
 
-def amg_tail(amg):
-    """First level of the V-cycle's shared launch (the number of operator levels if none)."""
-    ops = amg["levels"] - 1
-    return next((l for l in range(1, ops) if amg["rows"][l] <= TAIL_ROWS), ops)
+def step_launches(fam, n_prof, ni, scalars):
+    """How the linear solves of a step run, from the launches that n_prof profiled steps
+    made: (velocity, scalars, pressure, mass), each True where a solve is one launch."""
+    per = fam["resident_bicg"][0] / n_prof
+    return (per >= ni + scalars, scalars > 0 and per >= scalars, fam["resident_cg"][0] > 0, fam["mass"][0] == n_prof)
 
 
 def family_bytes(pb, nnz, args, tuning, amg):
@@ -193,6 +195,12 @@ def family_bytes(pb, nnz, args, tuning, amg):
                        (64 + 52 + 96) * N * D / 3 / 3, "(64 + 52 + 96) N / 3 per launch (D = 3)")
     out["assemble"] = ("k_ubar + k_cell_beta + k_assemble (convection assembly + Algorithm 2, once per step)",
                        60 * N + 80 * T + 12 * N + 48 * T + 28 * Z + 132 * N, "128 T + 28 Z + 204 N per step")
+    # solves that run as one launch: every array from memory once, whatever the iterations
+    # (they run on chip, bound by the latency of their grid-wide meetings)
+    out["resident_bicg"] = ("k_resident_bicg (a whole velocity or scalar solve)", 8 * Z + 4 * N + 24 * D * N + 4 * N,
+                            "8 Z + 24 D N + 8 N per solve")
+    out["resident_cg"] = ("k_resident_cg (a whole pressure solve)", 8 * Z + 8 * Z + 4 * N + 40 * N,
+                          "16 Z + 44 N per solve (multigrid operators not counted)")
     out["outer"] = ("k_bicg_outer(_rows) / k_pcg_outer_sell (float-float residuals of the sweeps)",
                     10 * Z + 84 * N, "(8 Z + 112 N + 12 Z + 56 N) / 2 per launch")
     if amg:
@@ -411,7 +419,7 @@ def run_ours(args, rank, world):
     tun_e = capi.oasis_get_tuning(run_e.solver)
     amg_info = capi.oasis_get_amg_info(run_e.solver) if pc == capi.OASIS_PC_AMG else None
     if amg_info:
-        amg_info["tail"] = amg_tail(amg_info)
+        amg_info["tail"] = amg_tail(amg_info, fam)
     run_e.close()
     if net_e is not None:
         net_e.close()
@@ -436,7 +444,8 @@ def run_ours(args, rank, world):
         if not n_l:
             continue
         ach = nbytes / (ms_l / n_l / 1e3) / 1e9
-        table[f] = {"kernel": kernel, "bound": "hbm", "algorithmic_bytes_per_launch": nbytes,
+        table[f] = {"kernel": kernel,
+                    "bound": "latency" if f.startswith("resident") else "hbm", "algorithmic_bytes_per_launch": nbytes,
                     "bytes_counted": per, "launches": n_l, "avg_launch_us": ms_l / n_l * 1e3,
                     "ms_per_step": ms_l / n_prof, "achieved": ach, "peak": peak, "unit": "GB/s",
                     "frac": ach / peak,
@@ -444,7 +453,7 @@ def run_ours(args, rank, world):
                     "traffic_source": MEASURED_TRAFFIC.get((args.workload, f + shape.get(f, "")), (None, None))[1]}
     # the dominant kernel: the single-kernel family (one kernel, one launch shape)
     # that takes the most time in the step
-    single = [f for f in ("pcg_spmv", "bicg_spmm", "amg_fine") if f in table]
+    single = [f for f in ("pcg_spmv", "bicg_spmm", "amg_fine", "resident_bicg", "resident_cg") if f in table]
     dominant = max(single, key=lambda f: table[f]["ms_per_step"])
     roofline = dict(table[dominant])
     roofline["family"] = dominant
@@ -528,8 +537,8 @@ def run_ours(args, rank, world):
     # and (all but the last) a correction, 5 per BiCGStab iteration; pressure: rhs
     # and guess 2, per sweep residual + CG start + (all but the last) correction,
     # 1 per CG iteration; update 1
-    # learned guess: input scales, inputs, two network layers, judge.  A solve small
-    # enough to be resident is one launch.  Multigrid: a V-cycle is 4 kernels per
+    # learned guess: input scales, inputs, two network layers, judge.  A solve that
+    # the profiled steps made as one launch is one.  Multigrid: a V-cycle is 4 kernels per
     # operator level before the shared launch + that (or the dense coarsest solve); per
     # sweep residual, start, V-cycle, product, update (and all but the last a
     # correction); per further iteration of an inner solve (every sweep but the
@@ -540,20 +549,20 @@ def run_ours(args, rank, world):
     # Scalars (approximate: the statistics give the largest iteration count):
     # assembly, two residual sweeps and a correction, 5 per BiCGStab iteration,
     # the final update.
+    one_u, one_c, one_p, one_m = step_launches(fam, n_prof, max(1, args.inner_iters), args.scalars)
     if amg_info:
         vk = 4 * amg_info["tail"] + 1
         p_kernels = sw_p * (5 + vk) + max(0, it_p - (sw_p - 1)) * (2 + vk)
     else:
         p_kernels = 3 * sw_p + it_p
     u_kernels = 2 * sw_u + 5 * it_u
-    small = pb.mesh.n_dofs <= RESIDENT_ROWS
-    if small:
+    if one_u:
         u_kernels = 1
-    if small and (not amg_info or run.nnz <= RESIDENT_AMG_ENTRIES):
+    if one_p:
         p_kernels = 3      # right-hand side, guess, solve
     ni = max(1, args.inner_iters)
-    upd_kernels = 3 + 2 * it_m if args.velocity_update == "consistent" else 1
-    upd_kernels += args.scalars * (5 + 5 * it_c)
+    upd_kernels = 1 if args.velocity_update != "consistent" else 2 if one_m else 3 + 2 * it_m
+    upd_kernels += args.scalars * (3 if one_c else 5 + 5 * it_c)
     n_asm = 2 if args.convection == "abe" else 3
     n_asm += 1   # the tentative velocity u^I formed once per dof for the pressure right-hand side
     launches = int(round(args.steps * (ni * (n_asm + u_kernels + p_kernels) + (ni - 1)
