@@ -80,10 +80,12 @@ struct AmgLevelDev {
 constexpr int64_t kSellMinRows = 65536;
 // Pattern entries up to which the multigrid pressure CG runs resident (one launch per
 // solve); in float64 fewer, its cycle moves twice the bytes.  Resident against separate
-// kernels, us per step at rtol 1e-8 / 1e-12 (pressure solve alone changed): 41^3 dofs,
-// 1.0 M entries: 1300 / 1519 mixed, 3132 / 3305 float64; 49^3, 1.7 M: 1705 / 1780
-// mixed; 57^3, 2.8 M: 2452 / 2032; 51^3 float64, 1.9 M: 6570 / 4893.
-constexpr int64_t kResidentAmgEntries = 1900000, kResidentAmgEntries64 = 1200000;
+// kernels, us per step at rtol 1e-8 / 1e-12 (pressure solve alone changed).  Mixed, cubes
+// of 0.92 / 1.15 / 1.41 / 1.71 M entries: 870 / 992, 996 / 1049, 1116 / 1092, 1192 / 1169;
+// triangles of 0.81 / 1.01 / 1.12 / 1.75 M (twice the rows per entry): 849 / 889, 893 /
+// 943, 979 / 964, 1326 / 1294.  Float64, cubes of 0.73 / 0.85 / 0.99 / 1.15 M: 2188 /
+// 2338, 2459 / 2484, 2629 / 2608, 3048 / 2866.
+constexpr int64_t kResidentAmgEntries = 1200000, kResidentAmgEntries64 = 900000;
 // The tail of a V-cycle of separate kernels, from the first coarser level with at most
 // this many rows down to the dense one and back, is one resident launch (resident.cu).
 // us per two steps with 20,000 / 40,000 / 60,000: 73x71x74 dofs float64 (level 1: 35k

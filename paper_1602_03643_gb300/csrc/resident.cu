@@ -1507,7 +1507,11 @@ ResidentPlan plan(const std::vector<int32_t>& row_ptr, int64_t n, int vectors, b
         p.blocks = blocks;
         return true;
     };
-    // all SMs, with at least 16 rows per block
+    // all SMs, with at least 16 rows per block.  us per step with 8 / 16 / 32 / 64: 289
+    // rows float64 multigrid 565 / 540 / 578 / 643, 1,089: 508 / 482 / 508 / 565 (mixed 350
+    // / 327 / 325 / 323), 512 float64 Jacobi 746 / 746 / 796 / 924, 2,197: 1099 / 1085 /
+    // 1122 / 1303 (mixed 502 / 490 / 505 / 527), 4,913 mixed multigrid 481 / 480 / 472 / 451
+    // (float64 948 / 951 / 949 / 1022).
     if (!shape((int)std::min<int64_t>(std::min(num_sms(), kResBlocks), (n + 15) / 16))) return p;
     // as many lanes per row as there are threads for
     constexpr int most = res_threads<P>();
@@ -1545,6 +1549,7 @@ void resident_set_wait(void* mem, int64_t cycles, cudaStream_t s) {
 
 template <class P, int D, int NR>
 ResidentPlan resident_plan_bicg(const std::vector<int32_t>& row_ptr, int64_t n) {
+    if (!P::mixed && NR > 1 && n > kResidentRows64) return {};
     const ResidentPlan pl = plan<P>(row_ptr, n, 6 * NR + 1);
     bool ok = pl.blocks > 0;
 #define OASIS_RES_FITS(G, M, ST) ok = ok && fits(k_resident_bicg<P, D, NR, G, M, ST>, pl)

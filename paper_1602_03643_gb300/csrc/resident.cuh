@@ -11,11 +11,17 @@ namespace oasis {
 constexpr int kResValues = 16;           // values of one grid-wide sum at most
 constexpr int kResBlocks = 1024;         // blocks of one launch at most
 // Rows up to which a solve may run resident (where a block's vectors fit its shared
-// memory: with three components about 440,000 rows mixed, 200,000 float64).  Resident
-// against separate kernels, us per step: 14x13x12 dofs float64 Jacobi eager 1160 / 4130;
-// 41^3 Jacobi mixed 1810 / 5690; 85^3 Jacobi mixed 16460 / 23330; velocity solve alone
-// changed: 73^3 mixed 2890 / 3140, 621^2 mixed 2070 / 2320.
-constexpr int64_t kResidentRows = 650000;
+// memory: three components to about 440,000 rows mixed; float64 one component to
+// 500,000, the mass solve of three to 240,000), and the d components of a float64
+// velocity solve together.  Resident against separate kernels, us per step, the named
+// solves alone changed.  Mixed: velocity 439,000 rows 5859 / 5920 (triangles 386,000: 1562
+// / 1796); one component at a time 636,000: 3520 / 5017; with two scalars 636,000: 4367 /
+// 4885; with the mass solve 493,000: 3365 / 3757; Jacobi pressure 636,000: 10009 / 12343.
+// Float64: velocity 132,700 rows 3683 / 3802, 148,900: 3905 / 3947, 185,200: 4736 / 4760,
+// 205,400: 5074 / 4913; triangles 90,600: 1513 / 1599, 160,800: 2287 / 2264; one component
+// at a time 357,900: 8427 / 9881; two scalars 357,900: 10116 / 10557; mass 205,400: 6840 /
+// 7217; Jacobi pressure 68,900: 4856 / 9233.
+constexpr int64_t kResidentRows = 650000, kResidentRows64 = 150000;
 
 // Device memory in which the blocks of a launch meet (zero between launches).
 struct ResidentSync {

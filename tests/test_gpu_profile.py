@@ -1,7 +1,8 @@
 """oasis_profile: eager steps run the same kernels with and without it (the same bits), and
 the families say which solves ran as one launch.  By sizes of rows and entries of K: every
-solve resident; multigrid pressure above the float64 limit of entries (box_44, 1.3 M); one
-component and scalars; forced shapes (separate kernels)."""
+solve resident; multigrid pressure above the limits of entries (box_44, 1.3 M) and between them
+(box_42, 1.1 M); a float64 velocity solve above its limit of rows; one component and scalars;
+forced shapes (separate kernels)."""
 import numpy as np
 import pytest
 
@@ -17,8 +18,10 @@ STEPS = 2
     (lambda: box3(9, 8, 10), 1, dict(pressure_pc=1), dict(bicg=1, cg=1)),
     (lambda: box3(9, 8, 10), 0, dict(pressure_pc=0), dict(bicg=1, cg=1)),
     (lambda: WP.taylor_green_2d(97), 0, dict(pressure_pc=1), dict(bicg=1, cg=1)),
-    (lambda: box3(44, 43, 45), 0, dict(pressure_pc=1), dict(bicg=1, cg=0)),
-    (lambda: box3(44, 43, 45), 1, dict(pressure_pc=1), dict(bicg=1, cg=1)),
+    (lambda: box3(44, 43, 45), 1, dict(pressure_pc=1), dict(bicg=1, cg=0)),
+    (lambda: box3(42, 41, 43), 0, dict(pressure_pc=1), dict(bicg=1, cg=0)),
+    (lambda: box3(42, 41, 43), 1, dict(pressure_pc=1), dict(bicg=1, cg=1)),
+    (lambda: box3(53, 52, 54), 0, dict(pressure_pc=1), dict(bicg=0, cg=0)),
     (lambda: WP.with_scalars(box3(14, 13, 12), ns=2), 1, dict(pressure_pc=1, velocity_update=1),
      dict(bicg=3, cg=1, mass=1)),
     (lambda: WP.with_scalars(box3(14, 13, 12), ns=2), 0, dict(pressure_pc=1, velocity_update=1, batch_rhs=0),

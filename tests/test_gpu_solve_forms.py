@@ -56,7 +56,8 @@ def test_nan(pc, precision, graph, forced):
         run.close()
 
 
-MESHES = {"square_190": lambda: WP.taylor_green_2d(190), "box_44": lambda: box3(44, 43, 45)}
+MESHES = {"square_190": lambda: WP.taylor_green_2d(190), "box_38": lambda: box3(38, 37, 39),
+          "box_44": lambda: box3(44, 43, 45)}
 
 
 @pytest.mark.parametrize("precision", [0, 1])
@@ -84,6 +85,7 @@ def test_options_in_both_forms(opts, name, precision):
                 one = launched_as_one(run)
                 assert one["resident_bicg"] == 2 * (ns + (pb.mesh.dim if opts.get("batch_rhs") == 0 else 1))
                 assert one["mass"] == (2 if opts.get("velocity_update") else 0)
+                assert one["resident_cg"] == (0 if name == "box_44" else 2)
             out.append(list(run.fields()[:2]) + ([run.scalar_fields()] if run.ns else []))
         finally:
             run.close()
