@@ -1513,8 +1513,15 @@ ResidentPlan plan(const std::vector<int32_t>& row_ptr, int64_t n, int vectors, b
     // 1122 / 1303 (mixed 502 / 490 / 505 / 527), 4,913 mixed multigrid 481 / 480 / 472 / 451
     // (float64 948 / 951 / 949 / 1022).
     if (!shape((int)std::min<int64_t>(std::min(num_sms(), kResBlocks), (n + 15) / 16))) return p;
-    // as many lanes per row as there are threads for
-    constexpr int most = res_threads<P>();
+    // As many lanes per row as there are threads for.  Where 256 threads have a group for
+    // every row the launch takes no more, half the registers of an SM, so that solves of
+    // solvers on other streams run beside it; larger systems take all of every SM.  15,625
+    // rows mixed multigrid, us per step and solver with 1 / 2 / 4 solvers stepped at once:
+    // 642 / 369 / 350 (512 threads 549 / 532 / 548, separate kernels 1111 / 611 / 353); one
+    // solver, 256 against 512 threads: 29,791 rows Jacobi 840 / 896, multigrid 751 / 732,
+    // 22,801 (triangles) 484 / 505, 8,000 float64 Jacobi 1504 / 1600, 4,913 float64
+    // multigrid 956 / 936.  68,921 rows with 256 threads: 1061 against 886 alone.
+    const int most = p.rows * (P::mixed ? 1 : 4) <= 256 ? 256 : res_threads<P>();
     p.lanes = 8;
     while (p.lanes > (P::mixed ? 1 : 4) && p.rows * p.lanes > most) p.lanes /= 2;
     p.threads = std::min(most, std::max(256, (p.rows * p.lanes + 31) / 32 * 32));
