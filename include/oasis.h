@@ -109,9 +109,9 @@ typedef struct oasis_params {
                               iteration, or the multigrid CG product with OASIS_PC_AMG):
                               0 = autotune at solver creation (every candidate timed on
                               this matrix, the fastest kept; where the system is small
-                              enough the whole pressure solve runs as one launch instead,
-                              which has no such shapes); k >= 1 = candidate k of
-                              oasis_get_tuning */
+                              enough the whole pressure solve runs as one launch instead
+                              ("One launch per solve" below), which has no such shapes);
+                              k >= 1 = candidate k of oasis_get_tuning */
     int32_t pressure_pc;   /* OASIS_PC_JACOBI or OASIS_PC_AMG (preconditioner of the
                               pressure CG) */
     int32_t inner_iters;   /* inner velocity/pressure iterations of Algorithm 1 (0 or 1 =
@@ -126,11 +126,21 @@ typedef struct oasis_params {
                               0 = autotune at solver creation (every candidate timed on this
                               mesh's pattern, the fastest kept; where the system is small
                               enough each velocity, scalar and mass solve runs as one launch
-                              instead, which has no such shapes); k >= 1 = candidate k of
-                              oasis_get_tuning's bicg_* fields.  The shapes add a row's
+                              instead ("One launch per solve" below), which has no such
+                              shapes); k >= 1 = candidate k of oasis_get_tuning's bicg_*
+                              fields.  The shapes add a row's
                               products in different orders: they agree to rounding, and a
                               solver keeps its shape for its life. */
 } oasis_params;
+
+/* One launch per solve.  A linear solve of a small system runs as one cooperative launch
+ * where the current device takes it (cooperative launches supported, all of its blocks
+ * resident); elsewhere, and where a shape is forced, as separate kernels.  With
+ * OASIS_PC_AMG the small levels of a V-cycle of separate kernels are one such launch as
+ * well, inside the conditional bodies of the captured step; not under MPS, which does not
+ * allow that.  The two forms agree to the solves' tolerances.  From about 39,000 rows on
+ * (OASIS_FP64: 9,700) such a launch fills every SM, so the solves of solvers that are
+ * stepped at once on streams of their own take turns there; separate kernels overlap. */
 
 /* Velocity update of the projection (Sec. 5).  LUMPED: u_k^n = u_k^I - dt
  * (dP^k phi) / ML, one pass.  CONSISTENT: M u_k^n = M u_k^I - dt dP^k phi with

@@ -15,13 +15,13 @@
 // The launch is cooperative: all blocks are resident, so every wait ends; each is
 // bounded all the same (OASIS_EWAIT).
 //
-// Bound by latency: a Jacobi CG iteration on 68,921 rows takes 5.0 us, of which the
-// meeting 1.0, the block's and the blocks' partial sums 0.5 + 1.0, the scalars 0.35 and
+// Bound by latency: a Jacobi CG iteration on 68,921 rows takes 5.3 us, of which the
+// meeting 1.0, the block's and the blocks' partial sums 0.5 + 1.0, the scalars 0.7 and
 // the product with its vector updates 2.1 (separate kernel: 15 us).  Whole steps, us,
-// separate kernels against resident: 1,089 dofs float64 multigrid 1500 / 585; 2,184
-// dofs float64 Jacobi, eager, host arrays 4020 / 1160; 68,921 mixed Jacobi 5830 / 1815;
-// 117,600 mixed multigrid with two scalars and the consistent-mass update 3040 / 1860;
-// 160,680 (triangles) mixed multigrid 2120 / 1365.  One thread per row (where there are
+// separate kernels against resident: 1,089 dofs float64 multigrid 1500 / 660; 2,184
+// dofs float64 Jacobi, eager, host arrays 4020 / 1230; 68,921 mixed Jacobi 5830 / 1900;
+// 117,600 with two scalars and the consistent-mass update (multigrid pressure separate)
+// 3040 / 1940; 160,680 (triangles) mixed multigrid 2120 / 1430.  One thread per row (where there are
 // rows enough for the threads) took 2.1 us in the product above where 4 lanes per row
 // took 3.5: fewer shuffles and a full warp in the row's vector updates.  Tried and
 // not kept: one 16-block cluster with its hardware barrier (0.3 us) for small systems

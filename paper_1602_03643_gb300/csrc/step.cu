@@ -864,7 +864,7 @@ static const BicgVariant<P, D>* bicg_variant_table() {
     } else {
         // No float64 shape caps its registers: for 5 blocks per SM they spilled 150-300
         // bytes, and steps with such a shape raised "misaligned address" (79,507 rows, 2
-        // lanes; the same step runs with each shape below).  Two rows in flight need fewer
+        // lanes; the same step runs with the shapes below that the tuner picks).  Two rows in flight need fewer
         // registers by themselves.  us per pair of products, capped / not: 79,507 rows 67.3
         // / 67.5, 132,651 rows 70.6 / 71.3; 4 lanes 75.4 / 71.1, 97.4 / 85.4.
         static const BicgVariant<P, D> t[kBicgVariants] = {
