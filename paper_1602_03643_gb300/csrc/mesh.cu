@@ -721,6 +721,13 @@ static void spmv_rows(const Mesh& m, const V* vals, const V* x, V* y, double* pa
 
 template <class V>
 static void spmv_launch(const Mesh& m, const V* vals, const V* x, V* y, int lanes, cudaStream_t s) {
+    // The library's choice: up to kRows16 rows 16 lanes each, whose rows are all in flight at
+    // once; above, few lanes and rows in flight per lane group.  us per product, 16 lanes /
+    // the other: float64 4,913 rows 4.1 / 8.2, 15,625: 6.2 / 8.2, 35,937: 10.3 / 8.2
+    // (triangles 3,721: 4.1 / 6.2, 22,801: 8.2 / 6.2); float32 35,937: 6.1 / 8.2, 117,649:
+    // 10.2 / 10.3 (triangles 22,801: 4.1 / 6.2, 90,601: 8.2 / 6.2).
+    constexpr int64_t kRows16 = sizeof(V) == 8 ? 16384 : 50000;
+    if (lanes == 0 && m.n <= kRows16) lanes = 16;
     if (lanes == 0) {
         spmv_rows<V, false>(m, vals, x, y, nullptr, nullptr, nullptr, s);
         return;

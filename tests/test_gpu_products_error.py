@@ -59,3 +59,25 @@ def test_own_shape_rounds_no_more_than_16_lanes(order):
             assert np.isfinite(a[~hit]).all()
     finally:
         c.oasis_mesh_destroy(h)
+
+
+@pytest.mark.parametrize("side,f64_own,f32_own", [(3, False, False), (24, False, False), (26, True, False),
+                                                  (37, True, True)])
+def test_small_products_take_16_lanes(side, f64_own, f32_own):
+    """Rows up to which the library's choice is 16 lanes per row: 16,384 float64, 50,000 float32
+    (the same bits as with lanes = 16; above, sums in another order)."""
+    import torch
+    from paper_1602_03643_gb300 import capi as c
+    m = WM.jitter_interior(WM.box_mesh_3d(side, side, side), 0.15, 1 / side, 3)
+    h = c.oasis_mesh_create(m.dim, m.coords, m.cells, m.dof_of_vertex, m.n_dofs, None)
+    try:
+        c.oasis_assemble_constant(h)
+        for dt, spmv, own in ((torch.float64, c.oasis_spmv_f64, f64_own), (torch.float32, c.oasis_spmv_f32, f32_own)):
+            x = torch.randn(m.n_dofs, dtype=dt, device="cuda", generator=torch.Generator("cuda").manual_seed(3))
+            y = [torch.empty_like(x) for _ in range(2)]
+            for out, lanes in zip(y, (0, 16)):
+                spmv(h, c.OASIS_MAT_K, x, out, lanes)
+            torch.cuda.synchronize()
+            assert torch.equal(y[0], y[1]) != own
+    finally:
+        c.oasis_mesh_destroy(h)
