@@ -24,6 +24,11 @@ int num_sms() {
     return sms;
 }
 
+// Partial sums of the stand-alone dot: one per 256 rows, and room for a resident wave.
+static int64_t dot_partials(int64_t n) {
+    return std::max<int64_t>((n + kBlock - 1) / kBlock, (int64_t)num_sms() * (2048 / kBlock));
+}
+
 int resident_blocks(const void* fn) {
     static std::mutex mu;
     static std::map<std::pair<int, const void*>, int> cache;
@@ -527,7 +532,7 @@ void assemble_constant(Mesh& m, cudaStream_t s) {
     OASIS_CUDA(cudaMemsetAsync(m.K64s.p, 0, m.n_sell * sizeof(double), s));
     OASIS_CUDA(cudaMemsetAsync(m.Kffs.p, 0, m.n_sell * sizeof(float2), s));
     k_csr_to_sell<<<grid_for(m.nnz), kBlock, 0, s>>>(m.nnz, m.sell_of_csr.p, m.K64.p, m.K64s.p, m.K32s.p, m.Kffs.p);
-    m.red_partial.alloc((size_t)((m.n + kBlock - 1) / kBlock));
+    m.red_partial.alloc((size_t)dot_partials(m.n));
     m.red_ticket.alloc(1);
     OASIS_CUDA(cudaMemsetAsync(m.red_ticket.p, 0, sizeof(uint32_t), s));
     OASIS_CUDA(cudaStreamSynchronize(s));
@@ -619,8 +624,8 @@ struct RowSum<float, NA> {
 // Bound by the dependent loads row pointer -> column -> operand, so rows in flight
 // count.  1,030,200 rows, 15.2 M entries in reverse Cuthill-McKee order, one product
 // each with M in float64, K in float32 and K in float64 with the dot: 393 us with 16
-// lanes per row and one row at a time (DOT: 256-row tiles through shared memory), 170
-// with this form (160 with one plain sum per lane, whose errors were 3 to 7 % larger than
+// lanes per row and one row at a time (DOT: 256-row tiles through shared memory), 156
+// with this form (four rows in flight for the dot as well: 170, and 160 with one plain sum per lane, whose errors were 3 to 7 % larger than
 // those of 16 lanes; 6.4e-8 against 3.9e-8 in float32); the bytes alone take 72 at the
 // copy rate.
 template <class V, int G, int U, bool C16, bool DOT>
@@ -706,16 +711,32 @@ static int wave_grid(const void* fn, int64_t n, int64_t rows) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)num_sms() * resident_blocks(fn)));
 }
 
+// Rows up to which the dot form takes 4 lanes per row and one row at a time; above, 2 lanes
+// and two rows: the fewer rows, the more blocks are needed to fill the chip, and the dot's
+// registers leave no more warps to four rows.  us per call (memset and launch ~5 of them)
+// with 4 x 1 / 2 x 2 / 2 x 4 (256-row tiles through shared memory, the form before these):
+// 1,331 rows 8.3 / 9.9 / 14.5 (12.4), 15,625: 9.9 / 10.3 / 14.9 (14.1), 24,389: 10.3 / 10.3
+// / 15.2 (13.1), 68,921: 16.5 / 12.3 / 16.4 (15.5), 274,625: 27.9 / 22.7 / 24.3 (30.8),
+// 1,030,301: - / 59.4 / 72.0; triangles 3,721: 8.2 / 8.5 / 10.9 (10.3), 36,481: 11.1 / 8.8 /
+// 12.4 (10.9), 63,001: 14.4 / 10.3 / 12.4 (12.3), 1,002,001: - / 34.5 / 35.8.
+constexpr int64_t kDotFew = 16384;
 template <class V, bool DOT>
 static void spmv_rows(const Mesh& m, const V* vals, const V* x, V* y, double* partial, uint32_t* ticket, double* xy,
                       cudaStream_t s) {
-    constexpr int G = 2, U = 4;
-    auto run = [&](auto fn) {
-        fn<<<wave_grid((const void*)fn, m.n, (int64_t)kBlock / G * U), kBlock, 0, s>>>(
-            m.n, m.row_ptr.p, m.col.p, m.csr_dcol.p, vals, x, y, partial, ticket, xy);
+    auto run = [&](auto fn, int64_t rows) {
+        // (no more blocks than partial sums)
+        const int grid = (int)std::min<int64_t>(wave_grid((const void*)fn, m.n, rows), dot_partials(m.n));
+        fn<<<grid, kBlock, 0, s>>>(m.n, m.row_ptr.p, m.col.p, m.csr_dcol.p, vals, x, y, partial, ticket, xy);
     };
-    if (m.csr_dcol.p) run(k_spmv_rows<V, G, U, true, DOT>);
-    else run(k_spmv_rows<V, G, U, false, DOT>);
+    auto shape = [&](auto lanes, auto in_flight) {
+        constexpr int G = decltype(lanes)::value, U = decltype(in_flight)::value;
+        if (m.csr_dcol.p) run(k_spmv_rows<V, G, U, true, DOT>, kBlock / G * U);
+        else run(k_spmv_rows<V, G, U, false, DOT>, kBlock / G * U);
+    };
+    using std::integral_constant;
+    if constexpr (!DOT) shape(integral_constant<int, 2>{}, integral_constant<int, 4>{});
+    else if (m.n <= kDotFew) shape(integral_constant<int, 4>{}, integral_constant<int, 1>{});
+    else shape(integral_constant<int, 2>{}, integral_constant<int, 2>{});
     OASIS_CUDA(cudaGetLastError());
 }
 
@@ -744,8 +765,7 @@ static void spmv_launch(const Mesh& m, const V* vals, const V* x, V* y, int lane
     OASIS_CUDA(cudaGetLastError());
 }
 
-// y = Mat x and x . y in float64; `partial` holds one double per block (at least one
-// per 256 rows, and never more blocks than that).
+// y = Mat x and x . y in float64; `partial` holds dot_partials(n) doubles, one per block.
 void spmv_dot_f64(const Mesh& m, const double* vals, const double* x, double* y, double* xy, double* partial,
                   uint32_t* ticket, cudaStream_t s) {
     OASIS_CUDA(cudaMemsetAsync(ticket, 0, sizeof(uint32_t), s));

@@ -81,3 +81,35 @@ def test_small_products_take_16_lanes(side, f64_own, f32_own):
             assert torch.equal(y[0], y[1]) != own
     finally:
         c.oasis_mesh_destroy(h)
+
+
+@pytest.mark.parametrize("side", [1, 2, 5, 24, 25, 40, 66])
+@pytest.mark.parametrize("order", ["natural", "random"])
+def test_dot_shapes(side, order):
+    """The dot form's shapes by rows (up to 16,384, above), with 16-bit columns and
+    without (random order from 33 per side on), down to fewer rows than a warp takes; scratch
+    for every block, of the mesh and of the form that allocates nothing."""
+    import torch
+    from paper_1602_03643_gb300 import capi as c
+    m = WM.box_mesh_3d(side, side, side)
+    perm = WM.random_permutation(m.n_dofs, 8) if order == "random" else np.arange(m.n_dofs, dtype=np.int32)
+    h = c.oasis_mesh_create(m.dim, m.coords, m.cells, m.dof_of_vertex, m.n_dofs, perm)
+    try:
+        c.oasis_assemble_constant(h)
+        rp, col = c.oasis_mesh_get_pattern(h)
+        v = c.oasis_mesh_get_matrix(h, c.OASIS_MAT_M)
+        x = np.random.default_rng(4).normal(size=m.n_dofs)
+        want = np.add.reduceat(v * x[col], rp[:-1])
+        xi = np.empty_like(x)
+        xi[perm] = x
+        X = torch.from_numpy(xi).cuda()
+        for call in (c.oasis_spmv_dot_f64, c.oasis_spmv_dot_f64_noalloc):
+            Y, d = torch.empty_like(X), torch.zeros(1, dtype=torch.float64, device="cuda")
+            for _ in range(2):                    # the ticket is left ready for the next call
+                call(h, c.OASIS_MAT_M, X, Y, d)
+            torch.cuda.synchronize()
+            # float64 sums of up to 15 positive and negative terms, and of all rows
+            assert np.abs(Y.cpu().numpy()[perm] - want).max() <= 1e-14 * np.abs(v).max() * np.abs(x).max() * 15
+            assert abs(float(d) - float(x @ want)) <= 1e-12 * float(np.abs(x) @ np.abs(want))
+    finally:
+        c.oasis_mesh_destroy(h)
